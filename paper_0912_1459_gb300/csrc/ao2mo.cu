@@ -45,9 +45,12 @@ struct StridedOut {
 
 // C[b] (m x n) = A[b] (m x k) * B[b] (k x n), all operands by strides.
 // A_M_CONTIG: A's unit stride is along m; B_N_CONTIG: B's unit stride is along n.
+// only_if (may be null): a device flag; the launch returns at once while it is 0.
 template <bool A_M_CONTIG, bool B_N_CONTIG, bool ACC = false>
 __global__ void __launch_bounds__(256)
-k_dgemm(int m, int n, int k, StridedMat A, StridedMat B, StridedOut C) {
+k_dgemm(int m, int n, int k, StridedMat A, StridedMat B, StridedOut C,
+        const int32_t* __restrict__ only_if) {
+    if (only_if && *only_if == 0) return;
     __shared__ double As[kGK][kGB + 1];
     __shared__ double Bs[kGK][kGB + 1];
     const int tid = threadIdx.x;
@@ -331,34 +334,34 @@ __global__ void k_gather_cols(const double* __restrict__ C, int32_t N, int32_t n
 
 template <bool AM, bool BN, bool ACC = false>
 static int launch_dgemm(int m, int n, int k, int batch, StridedMat A, StridedMat B, StridedOut C,
-                        cudaStream_t s) {
+                        cudaStream_t s, const int32_t* only_if = nullptr) {
     if (m <= 0 || n <= 0 || batch <= 0) return CDS_OK;
     dim3 grid((n + kGB - 1) / kGB, (m + kGB - 1) / kGB, batch);
-    k_dgemm<AM, BN, ACC><<<grid, 256, 0, s>>>(m, n, k, A, B, C);
+    k_dgemm<AM, BN, ACC><<<grid, 256, 0, s>>>(m, n, k, A, B, C, only_if);
     CDS_LAUNCH_CHECK();
     return CDS_OK;
 }
 
 // Strided-batched FP64 GEMM for other translation units; picks the load
 // pattern from the unit strides.  accumulate: C += A B (batch entries must
-// then write disjoint C).
+// then write disjoint C).  only_if: as k_dgemm.
 int launch_dgemm_strided(int m, int n, int k, int batch, const double* A, int64_t ars, int64_t acs,
                          int64_t abs_, const double* B, int64_t brs, int64_t bcs, int64_t bbs,
                          double* C, int64_t crs, int64_t ccs, int64_t cbs, cudaStream_t s,
-                         bool accumulate = false) {
+                         bool accumulate = false, const int32_t* only_if = nullptr) {
     StridedMat Am{A, ars, acs, abs_}, Bm{B, brs, bcs, bbs};
     StridedOut Cm{C, crs, ccs, cbs};
     const bool am = ars == 1, bn = bcs == 1;
     if (accumulate) {
-        if (am && bn) return launch_dgemm<true, true, true>(m, n, k, batch, Am, Bm, Cm, s);
-        if (am) return launch_dgemm<true, false, true>(m, n, k, batch, Am, Bm, Cm, s);
-        if (bn) return launch_dgemm<false, true, true>(m, n, k, batch, Am, Bm, Cm, s);
-        return launch_dgemm<false, false, true>(m, n, k, batch, Am, Bm, Cm, s);
+        if (am && bn) return launch_dgemm<true, true, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+        if (am) return launch_dgemm<true, false, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+        if (bn) return launch_dgemm<false, true, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+        return launch_dgemm<false, false, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
     }
-    if (am && bn) return launch_dgemm<true, true>(m, n, k, batch, Am, Bm, Cm, s);
-    if (am) return launch_dgemm<true, false>(m, n, k, batch, Am, Bm, Cm, s);
-    if (bn) return launch_dgemm<false, true>(m, n, k, batch, Am, Bm, Cm, s);
-    return launch_dgemm<false, false>(m, n, k, batch, Am, Bm, Cm, s);
+    if (am && bn) return launch_dgemm<true, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+    if (am) return launch_dgemm<true, false>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+    if (bn) return launch_dgemm<false, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+    return launch_dgemm<false, false>(m, n, k, batch, Am, Bm, Cm, s, only_if);
 }
 
 // U2[mu][b][nu] = L[K0+b][pair(mu,nu)] (vector index inside the row, so the

@@ -58,19 +58,22 @@ struct QpLayout {
     int32_t* active;
     int32_t* nactive;
     void* sigma_ws;
+    size_t sigma_bytes;
     size_t bytes;
 };
 
+// least: the smallest workspace the solve works in, else the one it asks for.
 static QpLayout qp_layout(void* ws, int32_t nmo, int32_t nocc, int32_t M, int32_t np,
-                          int32_t precision) {
+                          int32_t precision, bool least = false) {
     Carver c(ws);
     QpLayout l;
     l.sig = c.take<double>(np);
     l.dsig = c.take<double>(np);
     l.active = c.take<int32_t>(np);
     l.nactive = c.take<int32_t>(1);
-    size_t sw = sigma_ws_bytes(nmo, nocc, M, np, 1, precision);
-    l.sigma_ws = c.take<char>(sw);
+    l.sigma_bytes = least ? sigma_ws_min_bytes(nmo, nocc, M, np, 1, precision)
+                          : sigma_ws_bytes(nmo, nocc, M, np, 1, precision);
+    l.sigma_ws = c.take<char>(l.sigma_bytes);
     l.bytes = c.off;
     return l;
 }
@@ -97,6 +100,7 @@ extern "C" int cds_qp_solve(int32_t nmo, int32_t nocc, int32_t M, const double* 
     if (np == 0) return CDS_OK;
     if (!Lp || !orb || !eps || !omega || !pole || !iters || !status) return CDS_ERR_ARG;
     QpLayout lay = qp_layout(workspace, nmo, nocc, M, np, precision);
+    if (workspace_bytes < lay.bytes) lay = qp_layout(workspace, nmo, nocc, M, np, precision, true);
     if (!workspace || workspace_bytes < lay.bytes) return CDS_ERR_WORKSPACE;
     int nb = (np + 127) / 128;
     k_qp_init<<<nb, 128, 0, stream>>>(eps, orb, np, nmo, omega, pole, iters, status, lay.active,
@@ -106,7 +110,7 @@ extern "C" int cds_qp_solve(int32_t nmo, int32_t nocc, int32_t M, const double* 
     for (int32_t it = 0; it < max_iter && h_active > 0; ++it) {
         // the factors do not change during the solve: split them once
         int st = sigma2_dispatch(nmo, nocc, M, Lov, Lp, np, eps, omega, 1, precision, lay.active,
-                                 lay.sig, lay.dsig, lay.sigma_ws, stream, it == 0);
+                                 lay.sig, lay.dsig, lay.sigma_ws, lay.sigma_bytes, stream, it == 0);
         if (st) return st;
         CDS_CUDA_TRY(cudaMemsetAsync(lay.nactive, 0, sizeof(int32_t), stream));
         k_qp_step<<<nb, 128, 0, stream>>>(eps, orb, np, lay.sig, lay.dsig, conv, omega, pole,
@@ -316,6 +320,7 @@ extern "C" int cds_qp_solve_bracketed(int32_t nmo, int32_t nocc, int32_t M, cons
     if (!Lp || !orb || !eps || !omega || !pole || !iters || !status || !bracket)
         return CDS_ERR_ARG;
     QpLayout lay = qp_layout(workspace, nmo, nocc, M, np, precision);
+    if (workspace_bytes < lay.bytes) lay = qp_layout(workspace, nmo, nocc, M, np, precision, true);
     if (!workspace || workspace_bytes < lay.bytes) return CDS_ERR_WORKSPACE;
     int st = upload_brackets(nmo, nocc, np, orb, eps, bracket, stream);
     if (st) return st;
@@ -326,7 +331,7 @@ extern "C" int cds_qp_solve_bracketed(int32_t nmo, int32_t nocc, int32_t M, cons
     int32_t h_active = np;
     for (int32_t it = 0; it < max_iter && h_active > 0; ++it) {
         st = sigma2_dispatch(nmo, nocc, M, Lov, Lp, np, eps, omega, 1, precision, lay.active,
-                             lay.sig, lay.dsig, lay.sigma_ws, stream, it == 0);
+                             lay.sig, lay.dsig, lay.sigma_ws, lay.sigma_bytes, stream, it == 0);
         if (st) return st;
         CDS_CUDA_TRY(cudaMemsetAsync(lay.nactive, 0, sizeof(int32_t), stream));
         k_qp_step_bracketed<<<nb, 128, 0, stream>>>(eps, orb, np, lay.sig, lay.dsig, conv, omega,

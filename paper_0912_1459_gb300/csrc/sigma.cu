@@ -7,6 +7,7 @@
 // denominators in the same kernel; no o^2 v^2 integral array exists.
 #include "sigma.cuh"
 #include "sigma_tc.cuh"
+#include "sigma_x.cuh"
 
 namespace cds {
 
@@ -265,12 +266,15 @@ int sigma2_fp64(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const d
 }
 
 size_t fp64_cached_workspace_bytes(int32_t nmo, int32_t nocc, int32_t np) {
+    // two doubles per block of k_sigma_x, which has at most one block per item
     return fp64_part_bytes(nmo, nocc, np, 1);
 }
 
 int sigma2_cached_fp64(int32_t nmo, int32_t nocc, int32_t np, const double* eps, const double* E,
                        const int32_t* active, const double* cache, double* sigma, double* dsigma,
                        double* part, cudaStream_t stream) {
+    if (sigma_x_serves(nmo, nocc, np))
+        return sigma2_x_cached(nmo, nocc, np, eps, E, active, cache, sigma, dsigma, part, stream);
     SigmaTerm t0, t1;
     make_terms(nmo, nocc, 1, nullptr, nullptr, eps, t0, t1);
     const int64_t n0 = items_of(t0, np, kTB64), n1 = items_of(t1, np, kTB64);
@@ -357,24 +361,50 @@ static int mp2_fp64(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, con
     return sum_fixed(ep, nocc, e_total, stream);
 }
 
+static bool mp2_x_serves(int32_t nmo, int32_t nocc, int32_t M) {
+    return M > 0 && sigma_x_serves(nmo, nocc, nocc);
+}
+// per-orbital sums (when the caller wants none) and the workspace of mp2_x
+static size_t mp2_ws_x(int32_t nmo, int32_t nocc, int32_t M) {
+    return align_up((size_t)nocc * sizeof(double)) + mp2_x_bytes(nmo, nocc, M);
+}
+
 size_t sigma_ws_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
                       int32_t precision) {
-    if (precision == CDS_PREC_FP64) return fp64_part_bytes(nmo, nocc, np, nE);
+    if (precision == CDS_PREC_FP64) {
+        const size_t plain = fp64_part_bytes(nmo, nocc, np, nE);
+        return M > 0 && sigma_x_serves(nmo, nocc, np)
+                   ? std::max(plain, sigma_x_bytes(nmo, nocc, M, np, nE))
+                   : plain;
+    }
     if (is_split_tc(precision))
         return tc_workspace_bytes(nmo, nocc, M, np, nE, precision == CDS_PREC_TF32X3);
     return 0;
 }
 
+size_t sigma_ws_min_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
+                          int32_t precision) {
+    return precision == CDS_PREC_FP64 ? fp64_part_bytes(nmo, nocc, np, nE)
+                                      : sigma_ws_bytes(nmo, nocc, M, np, nE, precision);
+}
+
 int sigma2_dispatch(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* Lp,
                     int32_t np, const double* eps, const double* E, int32_t nE,
                     int32_t precision, const int32_t* active, double* sigma, double* dsigma,
-                    void* ws, cudaStream_t stream, bool resplit) {
-    if (precision == CDS_PREC_FP64)
+                    void* ws, size_t ws_bytes, cudaStream_t stream, bool resplit,
+                    void* cache) {
+    if (precision == CDS_PREC_FP64) {
+        // a workspace of the fused kernel's size is still served by that kernel
+        if (M > 0 && sigma_x_serves(nmo, nocc, np) &&
+            ws_bytes >= sigma_x_bytes(nmo, nocc, M, np, nE))
+            return sigma2_x(nmo, nocc, M, Lov, Lp, np, eps, E, nE, active, sigma, dsigma, ws,
+                            stream, resplit, static_cast<double*>(cache));
         return sigma2_fp64(nmo, nocc, M, Lov, Lp, np, eps, E, nE, active, sigma, dsigma,
-                           static_cast<double*>(ws), stream, nullptr);
+                           static_cast<double*>(ws), stream, static_cast<double*>(cache));
+    }
     if (is_split_tc(precision))
         return sigma2_tc(nmo, nocc, M, Lov, Lp, np, eps, E, nE, active, precision, sigma, dsigma,
-                         ws, stream, resplit);
+                         ws, stream, resplit, static_cast<float*>(cache));
     return CDS_ERR_UNSUPPORTED;
 }
 
@@ -402,15 +432,18 @@ extern "C" int cds_sigma2_diag(int32_t nmo, int32_t nocc, int32_t M, const doubl
     if (precision != CDS_PREC_FP64 && !is_split_tc(precision)) return CDS_ERR_UNSUPPORTED;
     if (np == 0) return CDS_OK;
     if (!Lp || !eps || !E || !sigma || (nocc > 0 && nocc < nmo && !Lov)) return CDS_ERR_ARG;
-    size_t need = sigma_ws_bytes(nmo, nocc, M, np, nE, precision);
+    size_t need = sigma_ws_min_bytes(nmo, nocc, M, np, nE, precision);
     if (need && (!workspace || workspace_bytes < need)) return CDS_ERR_WORKSPACE;
     return sigma2_dispatch(nmo, nocc, M, Lov, Lp, np, eps, E, nE, precision, nullptr, sigma,
-                           dsigma, workspace, stream);
+                           dsigma, workspace, workspace_bytes, stream);
 }
 
 extern "C" size_t cds_mp2_workspace_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t precision) {
     if (nmo <= 0 || nocc < 0 || nocc > nmo || M < 0) return 0;
-    if (precision == CDS_PREC_FP64) return mp2_fp64_bytes(nmo, nocc);
+    if (precision == CDS_PREC_FP64) {
+        const size_t plain = mp2_fp64_bytes(nmo, nocc);
+        return mp2_x_serves(nmo, nocc, M) ? std::max(plain, mp2_ws_x(nmo, nocc, M)) : plain;
+    }
     if (is_split16(precision)) return tc_mp2_workspace_bytes(nmo, nocc, M);
     return 0;
 }
@@ -427,10 +460,19 @@ extern "C" int cds_mp2_energy(int32_t nmo, int32_t nocc, int32_t M, const double
         if (e_total) CDS_CUDA_TRY(cudaMemsetAsync(e_total, 0, sizeof(double), stream));
         return CDS_OK;
     }
-    const size_t need = cds_mp2_workspace_bytes(nmo, nocc, M, precision);
+    const size_t need = precision == CDS_PREC_FP64
+                            ? mp2_fp64_bytes(nmo, nocc)
+                            : cds_mp2_workspace_bytes(nmo, nocc, M, precision);
     if (!workspace || workspace_bytes < need) return CDS_ERR_WORKSPACE;
-    if (precision == CDS_PREC_FP64)
+    if (precision == CDS_PREC_FP64) {
+        if (mp2_x_serves(nmo, nocc, M) && workspace_bytes >= mp2_ws_x(nmo, nocc, M)) {
+            double* ep = e_pair ? e_pair : static_cast<double*>(workspace);
+            char* ws = static_cast<char*>(workspace) + align_up((size_t)nocc * sizeof(double));
+            const int st = mp2_x(nmo, nocc, M, Lov, eps, ep, ws, stream);
+            return st ? st : sum_fixed(ep, nocc, e_total, stream);
+        }
         return mp2_fp64(nmo, nocc, M, Lov, eps, e_pair, e_total, workspace, stream);
+    }
     return mp2_tc(nmo, nocc, M, Lov, eps, precision, e_pair, e_total, workspace, stream);
 }
 
@@ -454,11 +496,8 @@ extern "C" int cds_sigma2_diag_cache(int32_t nmo, int32_t nocc, int32_t M, const
     if (!Lp || !eps || !E || !sigma || !cache || (nocc > 0 && nocc < nmo && !Lov))
         return CDS_ERR_ARG;
     if (cache_bytes < cds_sigma2_cache_bytes(nmo, nocc, np, precision)) return CDS_ERR_ARG;
-    size_t need = sigma_ws_bytes(nmo, nocc, M, np, nE, precision);
+    size_t need = sigma_ws_min_bytes(nmo, nocc, M, np, nE, precision);
     if (need && (!workspace || workspace_bytes < need)) return CDS_ERR_WORKSPACE;
-    if (precision == CDS_PREC_FP64)
-        return sigma2_fp64(nmo, nocc, M, Lov, Lp, np, eps, E, nE, nullptr, sigma, dsigma,
-                           static_cast<double*>(workspace), stream, static_cast<double*>(cache));
-    return sigma2_tc(nmo, nocc, M, Lov, Lp, np, eps, E, nE, nullptr, precision, sigma, dsigma,
-                     workspace, stream, true, static_cast<float*>(cache));
+    return sigma2_dispatch(nmo, nocc, M, Lov, Lp, np, eps, E, nE, precision, nullptr, sigma,
+                           dsigma, workspace, workspace_bytes, stream, true, cache);
 }

@@ -81,10 +81,14 @@ inline bool is_split_tc(int32_t precision) {
 
 size_t sigma_ws_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
                       int32_t precision);
+// The least workspace sigma2_dispatch works in (FP64: that of the fused kernel).
+size_t sigma_ws_min_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
+                          int32_t precision);
 
 int sigma2_dispatch(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* Lp,
                     int32_t np, const double* eps, const double* E, int32_t nE,
                     int32_t precision, const int32_t* active, double* sigma, double* dsigma,
-                    void* ws, cudaStream_t stream, bool resplit = true);
+                    void* ws, size_t ws_bytes, cudaStream_t stream, bool resplit = true,
+                    void* cache = nullptr);
 
 }  // namespace cds
