@@ -1,11 +1,14 @@
 // AO -> MO transform of the Cholesky vectors (paper Eq. transformation),
 // binary64:  B^K = C^T A^K C  with A^K the symmetric unpacked L^K.
 //
-// Per batch of kb vectors: unpack A^K (N x N), then two strided-batched FP64
-// GEMMs per output block,  T = C_occ^T A^K  (o x N)  and  Bov = T C_vir
-// (o x v), and the same for the requested orbital rows with C_P.  The second
-// GEMM writes straight into the K-innermost layouts Lov[i][a][K], Lp[t][r][K].
-// On this part FP64 issue rate, not HBM, bounds the transform.
+// Per batch of kb vectors: T[(r, K)][nu] = sum_mu C[mu][r] A^K[mu][nu] for the
+// occupied and the requested orbitals r together, then Lov = T_occ C_vir and
+// Lp = T_P C, written straight into the K-innermost layouts Lov[i][a][K], Lp[t][r][K].
+// The FP64 issue rate, not HBM, bounds these products on the FP64 units
+// (k_dchain, k_dgemm), so larger bases take them as exact-slice tensor-core
+// GEMMs (dgemm_tc.cu; kDxMinBasis, kDxChainBasis).  Measured, whole transform:
+// 240 functions (o = 40, 10 orbitals, M = 720) 23.2 ms on the FP64 units before;
+// 840 functions (o = 180, 8 orbitals, M = 240) 5.4 ms against 140 ms.
 //
 // F32X2 (double-FP32) form for the split-precision pipeline: every operand is
 // held as an (hi, lo) pair of floats (hi = fl32(x), lo = fl32(x - hi)) and
@@ -18,6 +21,8 @@
 
 #include "common.cuh"
 #include "ao2mo_tc.cuh"
+#include "dgemm_tc.cuh"
+#include "tcgen05.cuh"
 
 namespace cds {
 
@@ -309,19 +314,6 @@ __global__ void k_pair_cols_joint(const double* __restrict__ C, int32_t N, int32
                                 : make_float2(__int_as_float(0x7fc00000), 0.f);
 }
 
-// U[b][mu][nu] = L[K0+b][pair(mu,nu)]
-__global__ void k_unpack(const double* __restrict__ L, int64_t npair, int32_t K0, int32_t kb,
-                         int32_t N, double* __restrict__ U) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t per = (int64_t)N * N;
-    if (e >= per * kb) return;
-    int b = (int)(e / per);
-    int64_t r = e - b * per;
-    int mu = (int)(r / N), nu = (int)(r - (int64_t)mu * N);
-    int lo = min(mu, nu), hi = max(mu, nu);
-    U[e] = L[(int64_t)(K0 + b) * npair + (int64_t)hi * (hi + 1) / 2 + lo];
-}
-
 // Cp[mu][t] = C[mu][orb[t]]
 __global__ void k_gather_cols(const double* __restrict__ C, int32_t N, int32_t nmo,
                               const int32_t* __restrict__ orb, int32_t np, double* __restrict__ Cp) {
@@ -412,7 +404,6 @@ static int launch_dfgemm(int m, int n, int k, int batch, PairMat A, PairMat B, O
 struct AoLayout {
     double* U;    // [kb][N][N]             (float pairs in the F32X2 form)
     double* T;    // [kb][o + np][N]
-    double* Cp;   // [N][np]
     double* Cq;   // [N][nmo] float pairs of C (F32X2 form)
     double* Cj;   // [N][o + np] float pairs of C_occ and C_P (F32X2 form)
     size_t bytes;
@@ -423,7 +414,6 @@ static AoLayout ao_layout(void* ws, int32_t nbf, int32_t nmo, int32_t nocc, int3
     AoLayout l;
     l.U = c.take<double>((size_t)kAoBatch * nbf * nbf);
     l.T = c.take<double>((size_t)kAoBatch * std::max(nocc + np, 1) * nbf);
-    l.Cp = c.take<double>((size_t)nbf * std::max(np, 1));
     l.Cq = c.take<double>((size_t)nbf * nmo);
     l.Cj = c.take<double>((size_t)nbf * std::max(nocc + np, 1));
     l.bytes = c.off;
@@ -500,6 +490,240 @@ static int cd_to_mo_f32x2(int32_t N, int32_t nmo, int32_t nocc, int32_t M, const
     return CDS_OK;
 }
 
+// T[(r, K)][nu] = sum_mu C[mu][col(r)] A^K[mu][nu] on the FP64 units, one FMA chain
+// in mu order per element; rows r < nocc are the occupied columns, the others
+// the requested ones, vectors [K0, K0 + kb).  A block makes 4 RM rows and 64
+// columns of (K, nu), thread = (4 row groups, column).  The FP64 pipe (2 lanes a
+// clock and SM) bounds it whatever the operands come from, so the tile only
+// has to avoid idle lanes: rows in steps of 8, columns running on from one
+// vector to the next, the packed vectors read in place.  (The 64-row tiles of
+// k_dgemm, one launch each for the occupied and the requested rows, ran at 27 %
+// of the pipe for 40 + 10 rows of 240 functions.)
+template <int RM>
+__global__ void __launch_bounds__(256)
+k_dchain(const double* __restrict__ L, int64_t npair, int32_t N, int32_t K0, int32_t kb,
+         const double* __restrict__ C, int32_t nmo, int32_t nocc, const int32_t* __restrict__ orb,
+         int32_t r_first, int32_t r_end, double* __restrict__ T, const int32_t* __restrict__ only_if) {
+    if (only_if && *only_if == 0) return;
+    constexpr int R = 4 * RM;
+    __shared__ double As[kGK][R];
+    __shared__ double Bs[kGK][64];
+    const int tid = threadIdx.x, cl = tid & 63, rg = tid >> 6;
+    const int r0 = r_first + blockIdx.y * R;
+    const int64_t col0 = blockIdx.x * 64LL, ncols = (int64_t)kb * N;
+    double acc[RM] = {};
+    // this thread's column of B (four rows of a stage per thread)
+    const int64_t col = col0 + cl;
+    const int Kc = col < ncols ? (int)(col / N) : 0, nu = col < ncols ? (int)(col - (int64_t)Kc * N) : 0;
+    const double* Lk = L + (int64_t)(K0 + Kc) * npair;
+    for (int k0 = 0; k0 < N; k0 += kGK) {
+        for (int i = tid; i < kGK * R; i += 256) {
+            const int kk = i / R, r = r0 + i % R, mu = k0 + kk;
+            double v = 0.0;
+            if (r < r_end && mu < N) {
+                const int q = r < nocc ? r : orb[r - nocc];
+                v = q >= 0 && q < nmo ? C[(int64_t)mu * nmo + q]
+                                      : __longlong_as_double(0x7ff8000000000000LL);
+            }
+            As[kk][i % R] = v;
+        }
+#pragma unroll
+        for (int j = 0; j < kGK / 4; ++j) {
+            const int kk = rg + 4 * j, mu = k0 + kk;
+            const int hi = max(mu, nu), lo = min(mu, nu);
+            Bs[kk][cl] = col < ncols && mu < N ? Lk[(int64_t)hi * (hi + 1) / 2 + lo] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < kGK; ++kk) {
+            const double b = Bs[kk][cl];
+#pragma unroll
+            for (int i = 0; i < RM; ++i) acc[i] = fma(As[kk][rg + 4 * i], b, acc[i]);
+        }
+        __syncthreads();
+    }
+    if (col >= ncols) return;
+#pragma unroll
+    for (int i = 0; i < RM; ++i) {
+        const int r = r0 + rg + 4 * i;
+        if (r < r_end) T[(int64_t)r * ncols + col] = acc[i];
+    }
+}
+
+// Rows [r_first, r_end) of T in blocks of at most 64 rows, as even as they go.
+static int dchain(const double* L, int32_t N, int32_t K0, int32_t kb, const double* C, int32_t nmo,
+                  int32_t nocc, const int32_t* orb, int32_t r_first, int32_t r_end, double* T,
+                  const int32_t* only_if, cudaStream_t stream) {
+    const int rows = r_end - r_first;
+    if (rows <= 0 || kb <= 0) return CDS_OK;
+    const int nb = (rows + 63) / 64, rm = ((rows + nb - 1) / nb + 7) / 8 * 2;
+    const dim3 grid((unsigned)(((int64_t)kb * N + 63) / 64), (unsigned)((rows + 4 * rm - 1) / (4 * rm)));
+#define CDS_DCHAIN(RM_)                                                                          \
+    case RM_:                                                                                    \
+        k_dchain<RM_><<<grid, 256, 0, stream>>>(L, npair_of(N), N, K0, kb, C, nmo, nocc, orb,    \
+                                                r_first, r_end, T, only_if);                     \
+        break
+    switch (rm) {
+        CDS_DCHAIN(2);
+        CDS_DCHAIN(4);
+        CDS_DCHAIN(6);
+        CDS_DCHAIN(8);
+        CDS_DCHAIN(10);
+        CDS_DCHAIN(12);
+        CDS_DCHAIN(14);
+        default:
+            CDS_DCHAIN(16);
+    }
+#undef CDS_DCHAIN
+    CDS_LAUNCH_CHECK();
+    return CDS_OK;
+}
+
+// Lov[i][a][K0 + b] and Lp[t][r][K0 + b] from T on the FP64 units.
+static int fp64_second(int32_t N, int32_t nmo, int32_t nocc, int32_t np, const double* C, int32_t K0,
+                       int32_t kb, int32_t M, const double* T, double* Lov, double* Lp,
+                       const int32_t* only_if, cudaStream_t stream) {
+    const int32_t nv = nmo - nocc;
+    const int64_t trow = (int64_t)kb * N;
+    if (nocc > 0 && nv > 0) {
+        const int st = launch_dgemm<false, true>(
+            nocc, nv, N, kb, StridedMat{T, trow, 1, N}, StridedMat{C + nocc, nmo, 1, 0},
+            StridedOut{Lov + K0, (int64_t)nv * M, M, 1}, stream, only_if);
+        if (st) return st;
+    }
+    if (np > 0)
+        return launch_dgemm<false, true>(np, nmo, N, kb, StridedMat{T + nocc * trow, trow, 1, N},
+                                         StridedMat{C, nmo, 1, 0},
+                                         StridedOut{Lp + K0, (int64_t)nmo * M, M, 1}, stream,
+                                         only_if);
+    return CDS_OK;
+}
+
+// The least workspace every form works in (the FP64 products on the FP64 units).
+static size_t cd_to_mo_least_bytes(int32_t nbf, int32_t nmo, int32_t nocc, int32_t M, int32_t np) {
+    return std::max(ao_layout(nullptr, nbf, nmo, nocc, np).bytes,
+                    tr_any_workspace_bytes(nbf, nmo, nocc, np, tr_batch(nbf, std::max(M, 1))));
+}
+
+// Tensor-core products from this size on; smaller bases stay on the FP64 units.
+constexpr int kDxMinBasis = 32;
+// The first product keeps its FP64 FMA chain up to this size.  The exact-slice
+// product is the more accurate one (vectors of the 240-function ring, |C| up
+// to 294: Lov within 6e-13 of the exact transform, 2.4e-12 with the chain) and
+// an order of magnitude faster, but there the second product magnifies T's rounding
+// a hundredfold, and results of bases this small are held against a CPU's FP64
+// chain to 1e-11 of their largest entry, which only the same T can meet.
+constexpr int kDxChainBasis = 256;
+
+struct DxLayout {
+    dx::Operand cj, cv, ca;   // columns of C: occupied | requested, virtual, all
+    dx::Operand u, tov, tp;   // rows (K, nu) of the vectors, rows (i, K) and (t, K) of T
+    double* T;                // [(r, K)][nu]
+    int32_t* flag;            // [0] an operand is not finite, [1] error word
+    size_t bytes;
+};
+
+static DxLayout dx_layout(void* ws, int32_t N, int32_t nmo, int32_t nocc, int32_t np, int32_t kb) {
+    const int32_t nv = nmo - nocc;
+    // bulk copies want 16-byte addresses whatever the caller's workspace starts at
+    Carver c(ws ? (void*)align_up((size_t)ws) : nullptr);
+    DxLayout l;
+    const bool chain = N <= kDxChainBasis;
+    l.cj = dx::carve(c, 1, chain ? 0 : nocc + np, N, dx::kRowsB);
+    l.cv = dx::carve(c, 1, nv, N, dx::kRowsB);
+    l.ca = dx::carve(c, 1, nmo, N, dx::kRowsB);
+    l.u = dx::carve(c, 1, chain ? 0 : (int64_t)kb * N, N, dx::kRowsA);
+    l.tov = dx::carve(c, 1, (int64_t)kb * nocc, N, dx::kRowsA);
+    l.tp = dx::carve(c, 1, (int64_t)kb * np, N, dx::kRowsA);
+    l.T = c.take<double>((size_t)std::max(nocc + np, 1) * kb * N);
+    l.flag = c.take<int32_t>(2);
+    l.bytes = c.off + 256;
+    return l;
+}
+
+static bool dx_serves(int32_t nbf, int32_t nmo, int32_t nocc, int32_t np) {
+    return nbf >= kDxMinBasis && nbf <= (1 << 14) && nocc >= 0 && nocc <= nmo && nmo <= nbf &&
+           np >= 0 && np <= 65535 && tc::device_ok();
+}
+
+static int cd_to_mo_fp64(int32_t N, int32_t nmo, int32_t nocc, int32_t M, const double* L,
+                         const double* C, const int32_t* orb, int32_t np, double* Lov, double* Lp,
+                         void* ws, size_t ws_bytes, cudaStream_t stream) {
+    const int32_t nv = nmo - nocc;
+    const int32_t kbx = tr_batch(N, M);
+    // a workspace of the FP64-unit form's size is still served by that form
+    if (dx_serves(N, nmo, nocc, np) && ws_bytes >= dx_layout(nullptr, N, nmo, nocc, np, kbx).bytes) {
+        const DxLayout l = dx_layout(ws, N, nmo, nocc, np, kbx);
+        const bool ov = nocc > 0 && nv > 0;
+        int32_t *flag = l.flag, *err = l.flag + 1;
+        CDS_CUDA_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(int32_t), stream));
+        if (!ov && np == 0) return CDS_OK;
+        const bool chain = N <= kDxChainBasis;
+        const int32_t r0 = ov ? 0 : nocc;   // the occupied rows only when Lov is wanted
+        int st = CDS_OK;
+        if (!chain)
+            st = dx::slice_columns(dx::Columns{C, orb, nmo, nocc, 0}, l.cj, dx::kRowsB, N, flag, stream);
+        if (!st && ov)
+            st = dx::slice_columns(dx::Columns{C, nullptr, nmo, nmo, nocc}, l.cv, dx::kRowsB, N, flag,
+                                   stream);
+        if (!st && np > 0)
+            st = dx::slice_columns(dx::Columns{C, nullptr, nmo, nmo, 0}, l.ca, dx::kRowsB, N, flag,
+                                   stream);
+        if (st) return st;
+        const int64_t nocut = INT64_MAX;
+        for (int32_t K0 = 0; K0 < M; K0 += kbx) {
+            const int32_t kb = std::min(kbx, M - K0);
+            auto sized = [](dx::Operand o, int64_t rows, int R) {
+                o.per = rows;
+                o.per_pad = dx::padded_rows(rows, R);
+                return o;
+            };
+            const dx::Operand tov = sized(l.tov, (int64_t)kb * nocc, dx::kRowsA);
+            const dx::Operand tp = sized(l.tp, (int64_t)kb * np, dx::kRowsA);
+            const int64_t trow = (int64_t)kb * N;   // elements of T per r
+            if (!chain) {
+                const dx::Operand u = sized(l.u, (int64_t)kb * N, dx::kRowsA);
+                st = dx::slice_packed(dx::PackedRows{L, npair_of(N), K0, N}, u, dx::kRowsA, N, flag,
+                                      stream);
+                if (!st)
+                    st = dx::gemm(u, l.cj, 0, 1, dx::Out{l.T, nocut, 0, 1, 0, trow}, nullptr, flag, err,
+                                  stream);
+            }
+            // the FMA chain: always for the small bases, else for flagged operands
+            if (!st)
+                st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, l.T,
+                            chain ? nullptr : flag, stream);
+            if (!st && ov)
+                st = dx::slice_rows(dx::RowMajor{l.T, 0, N}, tov, dx::kRowsA, N, flag, stream);
+            if (!st && np > 0)
+                st = dx::slice_rows(dx::RowMajor{l.T + nocc * trow, 0, N}, tp, dx::kRowsA, N, flag,
+                                    stream);
+            if (!st && ov)
+                st = dx::gemm(tov, l.cv, 0, 1,
+                              dx::Out{Lov + K0, kb, (int64_t)nv * M, 1, 0, M}, nullptr, flag, err,
+                              stream);
+            if (!st && np > 0)
+                st = dx::gemm(tp, l.ca, 0, 1, dx::Out{Lp + K0, kb, (int64_t)nmo * M, 1, 0, M}, nullptr,
+                              flag, err, stream);
+            if (!st)
+                st = fp64_second(N, nmo, nocc, np, C, K0, kb, M, l.T, Lov, Lp, flag, stream);
+            if (st) return st;
+        }
+        if (ov && (st = dx::nan_on_error(err, Lov, (int64_t)nocc * nv * M, stream))) return st;
+        if (np > 0 && (st = dx::nan_on_error(err, Lp, (int64_t)np * nmo * M, stream))) return st;
+        return CDS_OK;
+    }
+    const AoLayout lay = ao_layout(ws, N, nmo, nocc, np);
+    const int32_t r0 = nocc > 0 && nv > 0 ? 0 : nocc;
+    for (int32_t K0 = 0; K0 < M; K0 += kAoBatch) {
+        const int32_t kb = std::min(kAoBatch, M - K0);
+        int st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, lay.T, nullptr, stream);
+        if (!st) st = fp64_second(N, nmo, nocc, np, C, K0, kb, M, lay.T, Lov, Lp, nullptr, stream);
+        if (st) return st;
+    }
+    return CDS_OK;
+}
+
 }  // namespace cds
 
 using namespace cds;
@@ -507,8 +731,11 @@ using namespace cds;
 extern "C" size_t cds_cd_to_mo_workspace_bytes(int32_t nbf, int32_t nmo, int32_t nocc, int32_t M,
                                             int32_t np) {
     if (nbf <= 0 || nocc < 0 || np < 0) return 0;
-    return std::max(ao_layout(nullptr, nbf, nmo, nocc, np).bytes,
-                    tr_any_workspace_bytes(nbf, nmo, nocc, np, tr_batch(nbf, std::max(M, 1))));
+    const size_t least = cd_to_mo_least_bytes(nbf, nmo, nocc, M, np);
+    return dx_serves(nbf, nmo, nocc, np)
+               ? std::max(least, dx_layout(nullptr, nbf, nmo, nocc, np,
+                                           tr_batch(nbf, std::max(M, 1))).bytes)
+               : least;
 }
 
 extern "C" int cds_cd_to_mo(int32_t nbf, int32_t nmo, int32_t nocc, int32_t M, const double* L,
@@ -521,7 +748,7 @@ extern "C" int cds_cd_to_mo(int32_t nbf, int32_t nmo, int32_t nocc, int32_t M, c
         return CDS_ERR_UNSUPPORTED;
     if (M == 0) return CDS_OK;
     if (!L || !C || !Lov || (np > 0 && (!orb || !Lp))) return CDS_ERR_ARG;
-    if (!workspace || workspace_bytes < cds_cd_to_mo_workspace_bytes(nbf, nmo, nocc, M, np))
+    if (!workspace || workspace_bytes < cd_to_mo_least_bytes(nbf, nmo, nocc, M, np))
         return CDS_ERR_WORKSPACE;
     if (is_tr_tc(precision)) {
         const int32_t kb = tr_batch(nbf, M);
@@ -535,44 +762,8 @@ extern "C" int cds_cd_to_mo(int32_t nbf, int32_t nmo, int32_t nocc, int32_t M, c
     AoLayout lay = ao_layout(workspace, nbf, nmo, nocc, np);
     if (precision == CDS_PREC_F32X2)
         return cd_to_mo_f32x2(nbf, nmo, nocc, M, L, C, orb, np, Lov, Lp, lay, stream);
-    const int64_t npair = npair_of(nbf);
-    const int32_t N = nbf, nv = nmo - nocc;
-    if (np > 0) {
-        k_gather_cols<<<(N * np + 255) / 256, 256, 0, stream>>>(C, N, nmo, orb, np, lay.Cp);
-        CDS_LAUNCH_CHECK();
-    }
-    for (int32_t K0 = 0; K0 < M; K0 += kAoBatch) {
-        int32_t kb = std::min(kAoBatch, M - K0);
-        int64_t tot = (int64_t)kb * N * N;
-        k_unpack<<<(unsigned)((tot + 255) / 256), 256, 0, stream>>>(L, npair, K0, kb, N, lay.U);
-        CDS_LAUNCH_CHECK();
-        StridedMat U{lay.U, N, 1, (int64_t)N * N};
-        if (nocc > 0 && nv > 0) {
-            // T[b][i][nu] = sum_mu C[mu][i] U[b][mu][nu]
-            StridedMat Aop{C, 1, nmo, 0};
-            StridedOut Tout{lay.T, N, 1, (int64_t)nocc * N};
-            int st = launch_dgemm<true, true>(nocc, N, N, kb, Aop, U, Tout, stream);
-            if (st) return st;
-            // Lov[i][a][K0+b] = sum_nu T[b][i][nu] C[nu][nocc+a]
-            StridedMat Top{lay.T, N, 1, (int64_t)nocc * N};
-            StridedMat Cv{C + nocc, nmo, 1, 0};
-            StridedOut Out{Lov + K0, (int64_t)nv * M, M, 1};
-            st = launch_dgemm<false, true>(nocc, nv, N, kb, Top, Cv, Out, stream);
-            if (st) return st;
-        }
-        if (np > 0) {
-            StridedMat Aop{lay.Cp, 1, np, 0};
-            StridedOut Tout{lay.T, N, 1, (int64_t)np * N};
-            int st = launch_dgemm<true, true>(np, N, N, kb, Aop, U, Tout, stream);
-            if (st) return st;
-            StridedMat Top{lay.T, N, 1, (int64_t)np * N};
-            StridedMat Call{C, nmo, 1, 0};
-            StridedOut Out{Lp + K0, (int64_t)nmo * M, M, 1};
-            st = launch_dgemm<false, true>(np, nmo, N, kb, Top, Call, Out, stream);
-            if (st) return st;
-        }
-    }
-    return CDS_OK;
+    return cd_to_mo_fp64(nbf, nmo, nocc, M, L, C, orb, np, Lov, Lp, workspace, workspace_bytes,
+                         stream);
 }
 
 // Adjoint of the transform: given dl/dLov and dl/dLp, dl/dC through
