@@ -979,28 +979,20 @@ k_cd_project_tc(int64_t n, const double* __restrict__ L, const float* __restrict
         tc_slice_item(it, itemsA, n, Lf, sigA, A, B, sigB, ctrl, k, s0, nseg);
 }
 
-// Step k, part 2: vector k, residuals, next pivot.  Five blocks per SM keep
-// the C60-shaped grid (690 blocks of 512 pairs) in one wave; the tensor-core
-// form runs on the screened pairs (425 blocks at C60), where four blocks per
-// SM do, and takes the registers (64) that its column and projection need.
-template <bool DF, bool SPEC, bool TC = false>
-__global__ void __launch_bounds__(kUpdThreads, TC ? 4 : 5)
+// Step k, part 2: vector k, residuals, next pivot (FP64 and float-pair forms).
+// Five blocks per SM keep the C60-shaped grid (690 blocks of 512 pairs) in one wave.
+template <bool DF, bool SPEC>
+__global__ void __launch_bounds__(kUpdThreads, 5)
 k_cd_update(int64_t n, int32_t k, int32_t max_rank, double* __restrict__ L,
             double* __restrict__ D, const uint8_t* __restrict__ cand,
             const double* __restrict__ ecol, const float2* __restrict__ G,
             double* __restrict__ blk_a, double* __restrict__ blk_b,
-            long long* __restrict__ blk_i, int32_t* __restrict__ piv, CdCtrl* ctrl,
-            PairF2 pf = PairF2{}) {
-    if constexpr (TC) {
-        pdl_trigger();
-        pdl_wait();
-    }
+            long long* __restrict__ blk_i, int32_t* __restrict__ piv, CdCtrl* ctrl) {
     if (ctrl->done) return;
-    if constexpr (TC) k = ctrl->kstep;   // the step number lives on the device (graph replays)
-    cd_step_body<DF, SPEC, TC>(n, k, max_rank, L, D, cand, ecol, G,
+    cd_step_body<DF, SPEC>(n, k, max_rank, L, D, cand, ecol, G,
                            reinterpret_cast<long long*>(blk_a),
                            reinterpret_cast<long long*>(blk_b), blk_i, piv, ctrl, blockIdx.x,
-                           gridDim.x, pf);
+                           gridDim.x);
 }
 
 // ---- screening of the tensor-core form (kScreenRel) ----
@@ -1092,16 +1084,29 @@ k_screen_gather(PairSoA pd, const double* __restrict__ D, const uint8_t* __restr
     }
 }
 
-// Rows [r0, r0 + nrows) of the compact vectors into the full rows of L (whose
-// screened entries were zeroed), as float pairs.
-__global__ void k_screen_scatter(const double* __restrict__ Lc, int64_t nc,
-                                 const int32_t* __restrict__ live, double* __restrict__ L,
-                                 int64_t n, int32_t r0, int32_t nrows) {
-    const int64_t total = (int64_t)nrows * nc;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = r0 + i / nc, j = i % nc;
-        L[r * n + live[j]] = Lc[r * nc + j];
+// inv[I] = compact index of pair I (inv preset to -1 elsewhere).
+__global__ void k_screen_inverse(const int32_t* __restrict__ live, int64_t nc,
+                                 int32_t* __restrict__ inv) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j < nc) inv[live[j]] = (int32_t)j;
+}
+
+// Rows [r0, r0 + gridDim.y) of the compact vectors into the full rows of L, screened
+// entries 0: as FP64, or (PAIRS) as the float pairs that the pipelined transform
+// reads.  Written whole, row by row, so L is neither zeroed before nor converted
+// after (zeroing, scattering and converting in place took 2.9 ms at 840 functions
+// and rank 899, this 0.8 ms).
+template <bool PAIRS>
+__global__ void __launch_bounds__(256)
+k_screen_spread(const float2* __restrict__ Lc, int64_t nc, const int32_t* __restrict__ inv,
+                double* __restrict__ L, int64_t n, int32_t r0) {
+    const int64_t r = r0 + (int64_t)blockIdx.y;
+    for (int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; I < n;
+         I += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t j = inv[I];
+        const float2 v = j >= 0 ? Lc[r * nc + j] : make_float2(0.f, 0.f);
+        if (PAIRS) reinterpret_cast<float2*>(L)[r * n + I] = v;
+        else L[r * n + I] = (double)v.x + (double)v.y;
     }
 }
 
@@ -1122,6 +1127,12 @@ __global__ void k_pairs_to_fp64(double* __restrict__ L, int64_t count) {
     const float2 v = reinterpret_cast<const float2*>(L)[i];
     L[i] = (double)v.x + (double)v.y;
 }
+
+}  // namespace cds
+
+#include "cd_steps.cuh"
+
+namespace cds {
 
 int pairs_to_fp64(double* L, int64_t count, cudaStream_t stream) {
     if (count <= 0) return CDS_OK;
@@ -1343,8 +1354,8 @@ static int cd_run_tc(int64_t n, int32_t max_rank, double* L, int32_t* piv, doubl
     int st = cd_tc_gemm_setup(&gemm, nc, lay.kcap, lay.A, lay.B, lay.sigA, lay.sigB, lay.G,
                               lay.ctrl, lay.err);
     if (st) return st;
-    // CUDA events around every GEMM launch of the steps that run (one pair per
-    // step of a host-check chunk, reused), summed after each check
+    // CUDA events around every GEMM launch (one pair per pass of a host-check
+    // chunk, reused), summed after each check
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CDS_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
     const bool timing = g_gemm_timing.on && cap == cudaStreamCaptureStatusNone;
@@ -1354,33 +1365,49 @@ static int cd_run_tc(int64_t n, int32_t max_rank, double* L, int32_t* piv, doubl
         ~EventGuard() { for (cudaEvent_t e : v) cudaEventDestroy(e); }
     } tev_guard{tev};
     if (timing)
-        for (int i = 0; i < 2 * kHostCheckEvery; ++i) {
+        for (int i = 0; i < 2 * kPassesPerCheck; ++i) {
             cudaEvent_t e;
             CDS_CUDA_TRY(cudaEventCreate(&e));
             tev.push_back(e);
         }
-    // the kernels of steps [k0, k1) (each reads its step number from ctrl)
-    auto enqueue = [&](int32_t k0, int32_t k1) -> int {
-        for (int32_t k = k0; k < k1; ++k) {
+    CdStepsArgs sa{};
+    sa.n = nc;
+    sa.nblk = nu;
+    sa.max_rank = max_rank;
+    sa.L = lay.Lc;
+    sa.D = lay.Dc;
+    sa.cand = lay.candc;
+    sa.G = lay.G;
+    sa.pf = lay.pf;
+    // two word sets of a 128-byte line per CTA and turn (at most one per block) in the
+    // memory of the float-pair form's integral column (4 KB per block)
+    sa.words[0] = reinterpret_cast<unsigned long long*>(lay.ecol);
+    sa.words[1] = sa.words[0] + 16 * (size_t)nu;
+    sa.piv = lay.pivc;
+    sa.ctrl = lay.ctrl;
+    sa.err = lay.err;
+    CDS_CUDA_TRY(cudaMemsetAsync(sa.words[0], 0, 32 * (size_t)nu * sizeof(unsigned long long), stream));
+    // `count` passes, each the slicing, the projection GEMM and the steps up to
+    // the next pass (everything reads its step from ctrl, and returns at once
+    // after the decomposition has stopped)
+    const int step_sms = pipe_tr_ctas() > 0 && pipe_tr_ctas() < nsm ? nsm - pipe_tr_ctas() : nsm;
+    auto enqueue = [&](int count) -> int {
+        for (int i = 0; i < count; ++i) {
             CDS_CUDA_TRY(launch_pdl(k_cd_project_tc, (unsigned)nres, kUpdThreads, 0, stream, nc,
                                     (const double*)lay.Lc, (const float*)lay.sigA, lay.A, lay.B,
                                     lay.sigB, (const CdCtrl*)lay.ctrl));
-            if (timing) CDS_CUDA_TRY(cudaEventRecord(tev[2 * (k - k0)], stream));
+            if (timing) CDS_CUDA_TRY(cudaEventRecord(tev[2 * i], stream));
             const int s2 = cd_tc_gemm_launch(gemm, stream);
             if (s2) return s2;
-            if (timing) CDS_CUDA_TRY(cudaEventRecord(tev[2 * (k - k0) + 1], stream));
-            CDS_CUDA_TRY(launch_pdl(k_cd_update<true, true, true>, (unsigned)nu, kUpdThreads, 0,
-                                    stream, nc, k, max_rank, lay.Lc, lay.Dc,
-                                    (const uint8_t*)lay.candc, (const double*)lay.ecol,
-                                    (const float2*)lay.G, lay.blk_a, lay.blk_b, lay.blk_i,
-                                    lay.pivc, lay.ctrl, lay.pf));
+            if (timing) CDS_CUDA_TRY(cudaEventRecord(tev[2 * i + 1], stream));
+            const int s3 = launch_steps(sa, step_sms, stream);
+            if (s3) return s3;
         }
         return CDS_OK;
     };
-    // a full chunk of steps as one CUDA graph, replayed at every host check
-    // (one launch instead of 3 x kHostCheckEvery): not under capture or
-    // timing, not on a default stream (no capture there), and only for
-    // decompositions long enough to repay the instantiation
+    // the passes between two host checks as one CUDA graph, replayed at every
+    // check: not under capture or timing, not on a default stream (no capture
+    // there), and only for decompositions long enough to repay the instantiation
     cudaGraphExec_t chunk = nullptr;
     struct ExecGuard {
         cudaGraphExec_t& e;
@@ -1390,10 +1417,10 @@ static int cd_run_tc(int64_t n, int32_t max_rank, double* L, int32_t* piv, doubl
     const bool default_stream =
         stream == nullptr || stream == cudaStreamLegacy || stream == cudaStreamPerThread;
     if (chunk_graph && !timing && cap == cudaStreamCaptureStatusNone && !default_stream &&
-        graph_min > 0 && max_rank >= std::max(graph_min, kHostCheckEvery)) {
+        graph_min > 0 && max_rank >= graph_min) {
         cudaGraph_t g = nullptr;
         CDS_CUDA_TRY(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-        const int s2 = enqueue(0, kHostCheckEvery);
+        const int s2 = enqueue(kPassesPerCheck);
         const cudaError_t ce = cudaStreamEndCapture(stream, &g);
         if (s2) {
             if (g) cudaGraphDestroy(g);
@@ -1404,37 +1431,59 @@ static int cd_run_tc(int64_t n, int32_t max_rank, double* L, int32_t* piv, doubl
         cudaGraphDestroy(g);
         CDS_CUDA_TRY(ie);
     }
+    // full rows: float pairs while a hook reads them or the caller converts them
+    const bool pairs_out = (on_chunk && *on_chunk) || !convert;
+    int32_t* inv = reinterpret_cast<int32_t*>(lay.pd.p);   // the pairs' FP64 data are not used any more
+    CDS_CUDA_TRY(cudaMemsetAsync(inv, 0xff, (size_t)n * sizeof(int32_t), stream));
+    k_screen_inverse<<<(unsigned)((nc + 255) / 256), 256, 0, stream>>>(lay.live, nc, inv);
+    CDS_LAUNCH_CHECK();
     CdCtrl h{};
-    for (int32_t k0 = 0; k0 <= max_rank; k0 += kHostCheckEvery) {
-        const int32_t k1 = std::min(max_rank, k0 + kHostCheckEvery);
-        if (chunk && k1 - k0 == kHostCheckEvery) {
+    int32_t rows = 0;
+    // a pass makes at least one step, so the rank cap bounds the loop
+    for (int32_t pass = 0; pass <= max_rank; pass += kPassesPerCheck) {
+        if (chunk) {
             CDS_CUDA_TRY(cudaGraphLaunch(chunk, stream));
-        } else if ((st = enqueue(k0, k1))) {
+        } else if ((st = enqueue(kPassesPerCheck))) {
             return st;
         }
-        count_launches(3ull * (unsigned long long)(k1 - k0));
-        if (k1 > k0) {   // this chunk's rows into L's full rows (screened entries 0)
-            CDS_CUDA_TRY(cudaMemsetAsync(L + (int64_t)k0 * n, 0,
-                                         (size_t)(k1 - k0) * n * sizeof(double), stream));
-            const int64_t items = (int64_t)(k1 - k0) * nc;
-            k_screen_scatter<<<(unsigned)std::min<int64_t>((items + 255) / 256, 8 * nsm), 256, 0,
-                               stream>>>(lay.Lc, nc, lay.live, L, n, k0, k1 - k0);
-            CDS_LAUNCH_CHECK();
-        }
+        count_launches(3ull * kPassesPerCheck);
         CDS_CUDA_TRY(cudaGetLastError());
+        const int32_t passes_before = std::max(h.passes, 1);   // the first one is counted at the start
         CDS_CUDA_TRY(cudaMemcpyAsync(&h, lay.ctrl, sizeof(CdCtrl), cudaMemcpyDeviceToHost, stream));
+        int32_t werr = 0;   // a bounded wait gave up: no step of this chunk is complete
+        CDS_CUDA_TRY(cudaMemcpyAsync(&werr, lay.err, sizeof(int32_t), cudaMemcpyDeviceToHost, stream));
         CDS_CUDA_TRY(cudaStreamSynchronize(stream));
-        if (timing) {   // the steps that ran (k < M once the decomposition has stopped)
-            const int32_t kr = h.done ? std::min(k1, h.M) : k1;
-            for (int32_t k = k0; k < kr; ++k) {
+        if (werr) return CDS_ERR_TIMEOUT;
+        if (timing) {   // the passes that ran
+            const int32_t ran = h.done ? std::min(h.passes - passes_before + 1, (int32_t)kPassesPerCheck)
+                                       : kPassesPerCheck;
+            for (int32_t i = 0; i < ran; ++i) {
                 float ms = 0.f;
-                CDS_CUDA_TRY(cudaEventElapsedTime(&ms, tev[2 * (k - k0)], tev[2 * (k - k0) + 1]));
+                CDS_CUDA_TRY(cudaEventElapsedTime(&ms, tev[2 * i], tev[2 * i + 1]));
                 g_gemm_timing.ms += ms;
                 ++g_gemm_timing.launches;
             }
         }
+        const int32_t made = h.done ? h.M : h.kstep;
+        if (made > rows) {   // the new rows into L's full rows
+            const dim3 sg((unsigned)std::min<int64_t>((n + 1023) / 1024, 4 * nsm), (unsigned)(made - rows));
+            const float2* Lcf = reinterpret_cast<const float2*>(lay.Lc);
+            if (pairs_out)
+                k_screen_spread<true><<<sg, 256, 0, stream>>>(Lcf, nc, inv, L, n, rows);
+            else
+                k_screen_spread<false><<<sg, 256, 0, stream>>>(Lcf, nc, inv, L, n, rows);
+            CDS_LAUNCH_CHECK();
+            rows = made;
+        }
         if (on_chunk && *on_chunk) {
-            st = (*on_chunk)(h.done ? h.M : k1, h.done != 0);
+            if (convert_after) {   // the hook's stream reads the rows just scattered
+                cudaEvent_t ev;
+                CDS_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+                CDS_CUDA_TRY(cudaEventRecord(ev, stream));
+                CDS_CUDA_TRY(cudaStreamWaitEvent(convert_after, ev, 0));
+                CDS_CUDA_TRY(cudaEventDestroy(ev));
+            }
+            st = (*on_chunk)(made, h.done != 0);
             if (st) return st;
         }
         if (h.done) break;
@@ -1445,7 +1494,7 @@ static int cd_run_tc(int64_t n, int32_t max_rank, double* L, int32_t* piv, doubl
     k_screen_finish<<<(unsigned)((fin + 255) / 256), 256, 0, stream>>>(lay.pivc, h.M, lay.live,
                                                                        piv, lay.Dc, nc, D);
     CDS_LAUNCH_CHECK();
-    if (h.M > 0 && convert) {
+    if (h.M > 0 && convert && pairs_out) {
         if (convert_after) {
             cudaEvent_t ev;
             CDS_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));

@@ -16,6 +16,7 @@ constexpr int kCdChunk = 2048;   // pivot row L^K_P staged in shared memory in c
 constexpr double kTieRel = 1e-12;
 constexpr double kNotPdRel = 1e-10;
 constexpr int kHostCheckEvery = 32;
+constexpr int kPassesPerCheck = 6;   // tensor-core form: streaming passes between host checks
 #ifndef CDS_KSPEC
 #define CDS_KSPEC 4
 #endif
@@ -76,7 +77,7 @@ struct CdCtrl {
     int32_t M;         // vectors produced
     int32_t _pad;
     unsigned int counter;  // last-block-done counter
-    unsigned int _pad2;
+    unsigned int _pad2;    // tensor-core form: arrivals at the tie scans' barrier
     // speculative projections (float-pair mode): the pivots of the current
     // batch's candidate set, the batch's first step, the slot of the current
     // pivot in the set, and whether this step streams L (a new batch)
@@ -90,7 +91,7 @@ struct CdCtrl {
     int32_t kdone;
     int32_t nlive;     // tensor-core form: pairs kept after screening
     int32_t kstep;     // tensor-core form: the step the kernels run next
-    int32_t _pad4;
+    int32_t _pad4;     // tensor-core form: tie scans so far
 };
 
 // Tensor-core form: pairs whose initial diagonal is below kScreenRel of the

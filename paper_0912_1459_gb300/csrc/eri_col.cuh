@@ -112,8 +112,13 @@ __device__ __forceinline__ PivotF2 pivot_f2(PairF2 pf, int64_t P) {
     return v;
 }
 
-// One element (rho_I|rho_P) of the column.
-__device__ __forceinline__ float2 eri_elem_df(PairF2 pf, int64_t I, const PivotF2& v) {
+// One element (rho_I|rho_P) of the column.  BS: row stride of the Taylor table
+// at boys (the global kBoysTaylorF2, or a caller's copy of its first rows in
+// shared memory, kBoysMidPoints rows).
+constexpr int kBoysMidPoints = (int)kMidT * kBoysPerUnit + 1;   // T < 16
+template <int BS = kBoysOrder>
+__device__ __forceinline__ float2 eri_elem_df(PairF2 pf, int64_t I, const PivotF2& v,
+                                              const float2* boys = &kBoysTaylorF2[0][0]) {
     const float2 pI = pf.p[I];
     const float2 dx = df_add(pf.Px[I], df_neg(v.qx));
     const float2 dy = df_add(pf.Py[I], df_neg(v.qy));
@@ -133,7 +138,7 @@ __device__ __forceinline__ float2 eri_elem_df(PairF2 pf, int64_t I, const PivotF
         const float2 T = df_mul(x, df_mul(rs, rs));
         const int i = min(max(__float2int_rn(T.x * (float)kBoysPerUnit), 0), kBoysPoints - 1);
         const float2 d = df_add(T, make_float2(-(float)i * (1.f / (float)kBoysPerUnit), 0.f));
-        const float2* c = kBoysTaylorF2[i];
+        const float2* c = boys + (BS == kBoysOrder ? i : min(i, kBoysMidPoints - 1)) * BS;
         float2 f = c[kBoysOrder - 1];
 #pragma unroll
         for (int m = kBoysOrder - 2; m >= 0; --m) f = df_add(df_mul(f, d), c[m]);
