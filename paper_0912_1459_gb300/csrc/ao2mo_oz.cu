@@ -292,19 +292,6 @@ __device__ __forceinline__ void pair_of(double x, float& f, float& r) {
 }
 
 // Operand row sources: element k of row `row` as a float pair.
-struct SrcPackedL {      // U rows (K, nu) over mu: A^K[nu][mu] from rows of L
-    const double* L;
-    const float2* Lf;
-    int64_t npair;
-    int32_t K0, N;
-    __device__ __forceinline__ void get(int64_t row, int k, float& f, float& r) const {
-        const int K = (int)(row / N), nu = (int)(row % N);
-        const int hi = max(k, nu), lo = min(k, nu);
-        const int64_t I = (int64_t)(K0 + K) * npair + (int64_t)hi * (hi + 1) / 2 + lo;
-        if (Lf) { const float2 v = Lf[I]; f = v.x; r = v.y; }
-        else pair_of(L[I], f, r);
-    }
-};
 struct SrcCols {         // row j over nu: C[nu][col(j)], col(j) = j < nocc ? j : orb[j - nocc] (orb may be null)
     const double* C;
     const int32_t* orb;
@@ -358,6 +345,144 @@ __global__ void __launch_bounds__(256) k_oz_slice(Src src, int64_t rows, int32_t
             const float v = ldexpf((float)(neg ? -d : d), -BETA * (s + 1));
             slices[s * plane + row * ld + k] = __float2bfloat16_rn(v);   // exact
         }
+    }
+}
+
+// q = trunc(f 2^(Q - e)) + trunc(r 2^(Q - e)) of the float pair (f, r), from the pair ...
+__device__ __forceinline__ long long fixed_of_pair(float f, float r, int e) {
+    return __float2ll_rz(ldexpf(f, QBITS - e)) + __float2ll_rz(ldexpf(r, QBITS - e));
+}
+// ... and from the double x whose pair it is (f = x rounded to 24 bits, r = the
+// remainder, of at most 29 bits, rounded to 24), in integer operations: the
+// conversions between double and float run on the FP64 pipe, two a clock and SM.
+// For |x| < 2^120 in a row whose largest entry is at least 2^-81 (entries below
+// FLT_MIN are then below one unit of q, and so are both parts of their pair).
+__device__ __forceinline__ long long fixed_of_double(double x, int e) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ffull);
+    if (ex == 0) return 0;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+    // x = m 2^(ex - 1075); f = F 2^29 units, r = R units
+    unsigned long long F = m >> 29;
+    const unsigned low = (unsigned)(m & 0x1fffffffull);
+    F += (low > 0x10000000u || (low == 0x10000000u && (F & 1ull))) ? 1ull : 0ull;
+    const int rem = (int)((long long)m - (long long)(F << 29));   // |rem| <= 2^28
+    unsigned ra = (unsigned)abs(rem);
+    const int drop = max(0, 8 - __clz((int)ra));                  // bits beyond 24
+    if (drop > 0) {
+        const unsigned half = 1u << (drop - 1), tail = ra & ((half << 1) - 1u);
+        ra >>= drop;
+        ra += (tail > half || (tail == half && (ra & 1u))) ? 1u : 0u;
+        ra <<= drop;
+    }
+    // units of q: shift by ex - 1075 + QBITS - e (negative or small)
+    const int sh = ex - 1075 + QBITS - e;
+    unsigned long long qf, qr;
+    const int sf = sh + 29;
+    if (sf >= 0) qf = F << sf;                 // f < 2^e: F 2^sf < 2^QBITS
+    else qf = sf > -64 ? F >> -sf : 0ull;
+    if (sh >= 0) qr = (unsigned long long)ra << sh;
+    else qr = sh > -32 ? (unsigned long long)(ra >> -sh) : 0ull;
+    const long long q = (long long)qf + (rem < 0 ? -(long long)qr : (long long)qr);
+    return (b >> 63) ? -q : q;
+}
+// Slice s of q as BF16 bits (exact; the float of a small integer through the low
+// bits of 1.5 2^23).
+__device__ __forceinline__ uint32_t slice_bits(long long q, int s) {
+    const bool neg = q < 0;
+    const unsigned long long aq = (unsigned long long)(neg ? -q : q);
+    const int d = (int)((aq >> (QBITS - BETA * (s + 1))) & 127ull);
+    const float f = __int_as_float(0x4B400000 + (neg ? -d : d)) - 12582912.f;
+    return __float_as_uint(f * __int_as_float((127 - BETA * (s + 1)) << 23)) >> 16;
+}
+
+// U rows (K, nu) over mu, A^K[nu][mu] from rows of L (FP64, or float pairs Lf): a block
+// slices eight neighbouring rows.  Right of the diagonal a row runs down a column
+// of the packed vector; eight neighbouring rows read 64 contiguous bytes of it per
+// mu, where one row at a time read 8 of every 32 bytes twice, once for the row
+// scale and once for the slices (8.1 ms of a 22.9 ms transform of 896 vectors of 840
+// functions, the conversions on the FP64 pipe included; 18.9 ms in all now).
+constexpr int kBand = 8;
+template <bool PAIRS>
+__global__ void __launch_bounds__(32 * kBand)
+k_oz_slice_packed(const double* __restrict__ L, const float2* __restrict__ Lf, int64_t npair,
+                  int32_t K0, int32_t N, int32_t bands, int64_t rows, int32_t ld,
+                  __nv_bfloat16* __restrict__ slices, float* __restrict__ scale) {
+    extern __shared__ double s_band[];      // [kBand][ldb]: doubles, or float pairs
+    const int ldb = N | 1;
+    const int K = blockIdx.x / bands, nu0 = (blockIdx.x % bands) * kBand;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double* src = (PAIRS ? reinterpret_cast<const double*>(Lf) : L) + (int64_t)(K0 + K) * npair;
+    const int nu = nu0 + w;
+    if (nu < N)      // left of the band and inside it: along the row
+        for (int mu = lane; mu < min(N, nu0 + kBand); mu += 32) {
+            const int hi = max(mu, nu), lo = min(mu, nu);
+            s_band[w * ldb + mu] = src[(int64_t)hi * (hi + 1) / 2 + lo];
+        }
+    // right of the band: eight lanes per mu, along nu
+    for (int mu = nu0 + kBand + (threadIdx.x >> 3); mu < N; mu += 4 * kBand) {
+        const int i = threadIdx.x & 7;
+        s_band[i * ldb + mu] = src[(int64_t)mu * (mu + 1) / 2 + nu0 + i];
+    }
+    __syncthreads();
+    if (nu >= N) return;
+    const double* row = s_band + w * ldb;
+    const int64_t orow = (int64_t)K * N + nu;
+    // the row scale: the power of two above the largest |f|
+    float mx = 0.f;
+    bool ints = false;
+    int e = 0;
+    if constexpr (PAIRS) {
+        for (int k = lane; k < N; k += 32) mx = fmaxf(mx, fabsf(reinterpret_cast<const float2*>(row)[k].x));
+#pragma unroll
+        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (mx > 0.f) frexpf(mx, &e);
+    } else {
+        unsigned long long m64 = 0;
+        for (int k = lane; k < N; k += 32) {
+            const unsigned long long a =
+                (unsigned long long)__double_as_longlong(row[k]) & 0x7fffffffffffffffull;
+            m64 = a > m64 ? a : m64;
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long x = __shfl_xor_sync(0xffffffffu, m64, o);
+            m64 = x > m64 ? x : m64;
+        }
+        const int ex = (int)(m64 >> 52) - 1023;     // the largest is in [2^ex, 2^(ex + 1))
+        ints = ex >= -81 && ex < 120;
+        if (ints) {
+            mx = (float)__longlong_as_double((long long)m64);
+            frexpf(mx, &e);
+        } else {   // zero, tiny, huge or NaN rows: through the float pair
+            for (int k = lane; k < N; k += 32) mx = fmaxf(mx, fabsf((float)row[k]));
+#pragma unroll
+            for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            if (mx > 0.f) frexpf(mx, &e);
+        }
+    }
+    if (lane == 0) scale[orow] = ldexpf(1.f, e);
+    const int64_t plane = rows * (int64_t)ld;
+    for (int k = 2 * lane; k < N; k += 64) {
+        long long q[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (k + j >= N) { q[j] = 0; continue; }
+            if constexpr (PAIRS) {
+                const float2 v = reinterpret_cast<const float2*>(row)[k + j];
+                q[j] = fixed_of_pair(v.x, v.y, e);
+            } else if (ints) {
+                q[j] = fixed_of_double(row[k + j], e);
+            } else {
+                float f, r;
+                pair_of(row[k + j], f, r);
+                q[j] = fixed_of_pair(f, r, e);
+            }
+        }
+        uint32_t* dst = reinterpret_cast<uint32_t*>(slices + orow * ld + k);   // ld, k even
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+            dst[s * (plane / 2)] = slice_bits(q[0], s) | (slice_bits(q[1], s) << 16);
     }
 }
 
@@ -453,6 +578,19 @@ int slice(const Src& src, int64_t rows, int32_t kdim, int32_t ld, __nv_bfloat16*
     return CDS_OK;
 }
 
+int slice_packed(const double* L, const float2* Lf, int32_t K0, int32_t kb, int32_t N, int32_t ld,
+                 __nv_bfloat16* out, float* scale, cudaStream_t stream) {
+    const int32_t bands = (N + kBand - 1) / kBand;
+    const size_t smem = (size_t)kBand * (N | 1) * sizeof(double);   // at most 67 KB (N <= MAX_K)
+    auto kern = Lf ? k_oz_slice_packed<true> : k_oz_slice_packed<false>;
+    if (smem > 48 * 1024)
+        CDS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<(unsigned)((int64_t)kb * bands), 32 * kBand, smem, stream>>>(
+        L, Lf, npair_of(N), K0, N, bands, (int64_t)kb * N, ld, out, scale);
+    CDS_LAUNCH_CHECK();
+    return CDS_OK;
+}
+
 }  // namespace oz
 
 size_t tr_oz_workspace_bytes(int32_t nbf, int32_t nmo, int32_t nocc, int32_t np, int32_t kb_max) {
@@ -480,7 +618,7 @@ int tr_oz_batch(int32_t nbf, int32_t nmo, int32_t nocc, int32_t np, const double
     const bool ov = nocc > 0 && nv > 0;
     if ((!ov && np == 0) || kb <= 0) return CDS_OK;
     const int64_t urows = (int64_t)kb * N, trows = (int64_t)nc * kb;
-    int st = oz::slice(oz::SrcPackedL{L, Lf, npair_of(N), K0, N}, urows, N, ld, l.u, l.u_s, stream);
+    int st = oz::slice_packed(L, Lf, K0, kb, N, ld, l.u, l.u_s, stream);
     if (st) return st;
     // GEMM 1: T^T[(K, nu)][r] -> T[(r, K)][nu] as float pairs
     st = oz::run_gemm(l.u, urows * ld, l.u_s, urows, l.cj, (int64_t)nc * ld, l.cj_s, nc, N, ld, N,
