@@ -97,75 +97,168 @@ struct GxArgs {
     void *ga_hi, *ga_lo, *gb_hi, *gb_lo;
 };
 
-// One 32 x 32 tile (x, c2) at fixed c1 per block: G in both layouts, the
-// energy partials and dSigma/dw of orbital t.
+// The BF16 split of x as split_d makes it, packed lo << 16 | hi, in integer
+// operations: f = x rounded to 24 bits, r = the remainder rounded to 24, hi =
+// bf16(f), lo = bf16((f - hi) + r).  The conversions it stands for run on the FP64
+// pipe, two a clock and SM.  False outside 2^-74 .. 2^126 (and for 0, inf, NaN).
+__device__ __forceinline__ bool split_bits(double x, uint32_t& packed) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ffull);
+    if ((unsigned)(ex - 949) > 200u) return false;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+    unsigned F = (unsigned)(m >> 29);
+    const unsigned low = (unsigned)m & 0x1fffffffu;
+    F += (low > 0x10000000u || (low == 0x10000000u && (F & 1u))) ? 1u : 0u;
+    int rem = (int)((unsigned)m - (F << 29));      // m - F 2^29, |rem| <= 2^28
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+    if (sign) rem = -rem;
+    const float f = __uint_as_float(sign | (((uint32_t)(ex - 896) << 23) + (F - 0x800000u)));
+    const float r = (float)rem * __int_as_float((ex - 948) << 23);
+    uint16_t h, l;
+    trc::split_bf16(f, r, h, l);
+    packed = (uint32_t)h | ((uint32_t)l << 16);
+    return true;
+}
+
+// 1 / d to within 1 ulp: the PTX reciprocal seed and one cubic Newton step; zero,
+// subnormal, infinite and NaN d take the plain division.
+__device__ __forceinline__ double recip(double d) {
+    const uint32_t ex = ((uint32_t)__double2hiint(d) >> 20) & 0x7ffu;
+    if (ex - 2u >= 2042u) return 1.0 / d;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    double e = fma(-d, r, 1.0);
+    e = fma(e, e, e);
+    return fma(r, e, r);
+}
+
+// Sums of four values over the warp (6 adds): lanes 8 i .. 8 i + 7 return value i.
+__device__ __forceinline__ double warp_sums4(const double (&v)[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool u = lane & 16, w = lane & 8;
+    double a = (u ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, u ? v[0] : v[2], 16);
+    double b = (u ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, u ? v[1] : v[3], 16);
+    a = (w ? b : a) + __shfl_xor_sync(0xffffffffu, w ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+// 32 x 32 tiles (x, c2) of up to kC1 values of c1 in turn: G in both layouts, the
+// energy partials and dSigma/dw of orbital t.  The FP64 pipe bounds it: about 11
+// operations per element here (8 for D, its reciprocal, G and r, 2.4 for the sums
+// over x, c2 and c1, which meet across the warp once per kC1 tiles), 60 with
+// divisions, a warp sum per row and the splits' conversions on that pipe too
+// (60.6 ms of an
+// 80.2 ms gradient of 8 orbitals of 840 functions; 39.7 ms in all now).
+constexpr int kC1 = 4;
 template <bool TF32>
 __global__ void __launch_bounds__(256)
 k_adj_gx(GxArgs a, int32_t t, int32_t nmo, const double* __restrict__ eps,
          const double* __restrict__ omega, double* __restrict__ deps_t,
          double* __restrict__ dsig_t) {
-    __shared__ double sY[kT][kT + 1], sP[kT][kT + 1], sG[kT][kT + 1];
-    __shared__ double rx[kT], rc2[kT], rc1;
+    __shared__ double sP[kT][kT + 1];
+    __shared__ E<TF32> sH[kT][kT + 1], sL[kT][kT + 1];
+    __shared__ double rx[kT], rc2[kT], rc1[kC1], sa[kT];
     const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    const int32_t c2_0 = blockIdx.x * kT, x0 = blockIdx.y * kT, c1 = blockIdx.z;
-    const int64_t col0 = (int64_t)c1 * a.n2;
-    if (ty == 0) { rx[tx] = 0.0; rc2[tx] = 0.0; }
-    if (tx == 0 && ty == 0) rc1 = 0.0;
-    for (int i = ty; i < kT; i += 8) {
-        const int32_t x = x0 + i, c2 = c2_0 + tx;
-        const bool ok = x < a.nx && c2 < a.n2;
-        sY[i][tx] = ok ? a.X[(int64_t)x * a.ldc + col0 + c2] : 0.0;
-        if (a.swap_c1) {
-            sP[i][tx] = ok ? a.X[(int64_t)c1 * a.ldc + (int64_t)x * a.n2 + c2] : 0.0;
-        } else {   // partner X[c2][c1 n2 + x]: rows c2, read along x, stored transposed
-            const int32_t cr = c2_0 + i, xr = x0 + tx;
-            sP[tx][i] = (cr < a.n2 && xr < a.nx) ? a.X[(int64_t)cr * a.ldc + col0 + xr] : 0.0;
-        }
-    }
-    __syncthreads();
+    const int32_t c2_0 = blockIdx.x * kT, x0 = blockIdx.y * kT, c1_0 = blockIdx.z * kC1;
+    const int32_t nc1 = min(kC1, a.n1 - c1_0);
     const double w = omega[t];
     const double sgn = a.swap_c1 ? 1.0 : -1.0;   // D = w - e_x + sgn (e_c2 - e_c1)
-    const double ec1 = eps[c1];
+    if (ty == 0) {
+        rx[tx] = 0.0;
+        rc2[tx] = 0.0;
+        sa[tx] = x0 + tx < a.nx ? w - eps[a.xoff + x0 + tx] : 0.0;
+        if (tx < kC1) rc1[tx] = 0.0;
+    }
+    const bool cok = c2_0 + tx < a.n2;
+    const double ec2 = cok ? eps[a.nocc + c2_0 + tx] : 0.0;
     E<TF32>* gah = (E<TF32>*)a.ga_hi;
     E<TF32>* gal = (E<TF32>*)a.ga_lo;
-    double rsum = 0.0, rcol = 0.0;
-    for (int i = ty; i < kT; i += 8) {   // one warp per row x of the tile
-        const int32_t x = x0 + i, c2 = c2_0 + tx;
-        double G = 0.0, r = 0.0;
-        if (x < a.nx && c2 < a.n2) {
-            const double y = sY[i][tx], yx = sP[i][tx];
-            const double D = w - eps[a.xoff + x] + sgn * (eps[a.nocc + c2] - ec1);
-            G = (4.0 * y - 2.0 * yx) / D;
-            r = (2.0 * y - yx) * y / (D * D);
-            split_d<TF32>(G, gah, gal, ((int64_t)a.tl * a.nx + x) * a.ldc + col0 + c2);
-        }
-        sG[i][tx] = G;
-        rcol += r;
-        double rrow = r;
-        for (int o = 16; o; o >>= 1) rrow += __shfl_xor_sync(0xffffffffu, rrow, o);
-        if (tx == 0) rx[i] = rrow;
-        rsum += rrow;
-    }
-    atomicAdd(&rc2[tx], rcol);
-    if (tx == 0) atomicAdd(&rc1, rsum);
-    __syncthreads();
-    // GB[(c1, c2)][(tl, x)]: 32 consecutive x per warp store
     E<TF32>* gbh = (E<TF32>*)a.gb_hi;
     E<TF32>* gbl = (E<TF32>*)a.gb_lo;
-    for (int i = ty; i < kT; i += 8) {
-        const int32_t c2 = c2_0 + i, x = x0 + tx;
-        if (c2 < a.n2 && x < a.nx)
-            split_d<TF32>(sG[tx][i], gbh, gbl,
-                          (col0 + c2) * a.ldk + (int64_t)a.tl * a.nx + x);
+    double rr[4] = {}, rcol = 0.0, rt[kC1] = {};
+#pragma unroll
+    for (int u = 0; u < kC1; ++u) {
+        if (u >= nc1) break;                     // the same in the whole block
+        const int32_t c1 = c1_0 + u;
+        const int64_t col0 = (int64_t)c1 * a.n2;
+        double y[4], yx[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = ty + 8 * q;
+            const int32_t x = x0 + i, c2 = c2_0 + tx;
+            const bool ok = x < a.nx && cok;
+            y[q] = ok ? a.X[(int64_t)x * a.ldc + col0 + c2] : 0.0;
+            if (a.swap_c1) {
+                yx[q] = ok ? a.X[(int64_t)c1 * a.ldc + (int64_t)x * a.n2 + c2] : 0.0;
+            } else {   // partner X[c2][c1 n2 + x]: rows c2, read along x, stored transposed
+                const int32_t cr = c2_0 + i, xr = x0 + tx;
+                sP[tx][i] = (cr < a.n2 && xr < a.nx) ? a.X[(int64_t)cr * a.ldc + col0 + xr] : 0.0;
+            }
+        }
+        __syncthreads();                         // sP, sa; the previous tile's sH, sL are read
+        const double bt = sgn * (ec2 - eps[c1]);
+        double rsum = 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = ty + 8 * q;
+            const int32_t x = x0 + i;
+            const bool ok = x < a.nx && cok;
+            const double p = a.swap_c1 ? yx[q] : sP[i][tx];
+            double G = 0.0, r = 0.0;
+            if (ok) {
+                const double rc = recip(sa[i] + bt);
+                const double n = fma(2.0, y[q], -p);   // 2 X - X_partner
+                const double h = n * rc;
+                G = 2.0 * h;
+                r = h * (y[q] * rc);
+                uint32_t pk;
+                if constexpr (TF32) {
+                    split_d<TF32>(G, &sH[i][tx], &sL[i][tx], 0);
+                } else if (split_bits(G, pk)) {
+                    sH[i][tx] = (uint16_t)pk;
+                    sL[i][tx] = (uint16_t)(pk >> 16);
+                } else {
+                    split_d<TF32>(G, &sH[i][tx], &sL[i][tx], 0);
+                }
+                const int64_t e = ((int64_t)a.tl * a.nx + x) * a.ldc + col0 + c2_0 + tx;
+                gah[e] = sH[i][tx];
+                gal[e] = sL[i][tx];
+            }
+            rr[q] += r;
+            rsum += r;
+        }
+        rcol += rsum;
+        rt[u] = rsum;
+        __syncthreads();
+        // GB[(c1, c2)][(tl, x)]: 32 consecutive x per warp store
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = ty + 8 * q;
+            const int32_t c2 = c2_0 + i, x = x0 + tx;
+            if (c2 < a.n2 && x < a.nx) {
+                const int64_t e = (col0 + c2) * a.ldk + (int64_t)a.tl * a.nx + x;
+                gbh[e] = sH[tx][i];
+                gbl[e] = sL[tx][i];
+            }
+        }
     }
+    const double srow = warp_sums4(rr), sc1 = warp_sums4(rt);
+    if ((tx & 7) == 0) {
+        rx[ty + 8 * (tx >> 3)] = srow;           // each row belongs to one warp
+        atomicAdd(&rc1[tx >> 3], sc1);
+    }
+    atomicAdd(&rc2[tx], rcol);
+    __syncthreads();
     double* de = deps_t + (int64_t)t * nmo;
     if (ty == 0) {
         if (x0 + tx < a.nx) atomicAdd(de + a.xoff + x0 + tx, rx[tx]);
         if (c2_0 + tx < a.n2) atomicAdd(de + a.nocc + c2_0 + tx, -sgn * rc2[tx]);
     }
-    if (tx == 0 && ty == 1) {
-        atomicAdd(de + c1, sgn * rc1);
-        atomicAdd(dsig_t + t, -rc1);
+    if (ty == 1 && tx < nc1) {
+        atomicAdd(de + c1_0 + tx, sgn * rc1[tx]);
+        atomicAdd(dsig_t + t, -rc1[tx]);
     }
 }
 
@@ -288,7 +381,8 @@ int gradient(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const doub
                 a.ga_lo = sum == 0 ? l.ga1_lo : l.ga2_lo;
                 a.gb_hi = sum == 0 ? l.gb1_hi : l.gb2_hi;
                 a.gb_lo = sum == 0 ? l.gb1_lo : l.gb2_lo;
-                dim3 grid((unsigned)((v + kT - 1) / kT), (unsigned)((nx + kT - 1) / kT), (unsigned)o);
+                dim3 grid((unsigned)((v + kT - 1) / kT), (unsigned)((nx + kT - 1) / kT),
+                          (unsigned)((o + kC1 - 1) / kC1));
                 k_adj_gx<TF32><<<grid, dim3(kT, 8), 0, stream>>>(a, t, nmo, eps, omega, l.deps_t,
                                                                   l.dsig_t);
                 CDS_LAUNCH_CHECK();
