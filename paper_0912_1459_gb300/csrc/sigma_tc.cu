@@ -576,28 +576,71 @@ __device__ __forceinline__ double split_scale(const unsigned long long* amax, bo
     return ldexp(1.0, ex - 1);
 }
 
-// hi = r(s x), lo = r(s x - hi) in bf16 or fp16; columns J >= M are zero.
+// hi = bf16(x) and lo = bf16(x - hi), rounded to nearest (ties to even), in integer
+// operations: conversions from double run on the FP64 pipe, two a clock and SM.
+// False where an exponent leaves the normal range (and for 0, inf, NaN).
+__device__ __forceinline__ bool split_bf16_bits(double x, uint32_t& hi, uint32_t& lo) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ffull);
+    if ((unsigned)(ex - 960) > 180u) return false;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+    const uint32_t sign = (uint32_t)(b >> 48) & 0x8000u;
+    unsigned h = (unsigned)(m >> 45);                       // 8 bits
+    const unsigned long long tail = m & ((1ull << 45) - 1), half = 1ull << 44;
+    h += (tail > half || (tail == half && (h & 1u))) ? 1u : 0u;
+    hi = sign | (((uint32_t)(ex - 896) << 7) + (h - 128u));
+    const long long rem = (long long)(m - ((unsigned long long)h << 45));   // |rem| <= 2^44
+    if (rem == 0) { lo = 0; return true; }
+    const unsigned long long a = (unsigned long long)(rem < 0 ? -rem : rem);
+    const int lead = 63 - __clzll((long long)a);
+    unsigned l;
+    if (lead >= 8) {
+        const int drop = lead - 7;
+        l = (unsigned)(a >> drop);
+        const unsigned long long t2 = a & ((1ull << drop) - 1), h2 = 1ull << (drop - 1);
+        l += (t2 > h2 || (t2 == h2 && (l & 1u))) ? 1u : 0u;
+    } else {
+        l = (unsigned)a << (7 - lead);
+    }
+    lo = (sign ^ (rem < 0 ? 0x8000u : 0u)) | (((uint32_t)(ex - 896 - 52 + lead) << 7) + (l - 128u));
+    return true;
+}
+
+// hi = r(s x), lo = r(s x - hi) in bf16 or fp16; columns J >= M are zero.  One warp
+// per row, two columns per lane.
 template <typename T>
-__global__ void k_split16(const double* __restrict__ src, int64_t rows, int32_t M, int32_t Mp,
-                          const unsigned long long* __restrict__ amax, T* __restrict__ hi,
-                          T* __restrict__ lo) {
+__global__ void __launch_bounds__(256)
+k_split16(const double* __restrict__ src, int64_t rows, int32_t M, int32_t Mp,
+          const unsigned long long* __restrict__ amax, T* __restrict__ hi, T* __restrict__ lo) {
     constexpr bool BF16 = std::is_same<T, __nv_bfloat16>::value;
     const double sc = split_scale(amax, BF16);
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= rows * Mp) return;
-    int64_t r = e / Mp;
-    int J = (int)(e - r * Mp);
-    double x = J < M ? src[r * M + J] * sc : 0.0;
-    if constexpr (BF16) {
-        __nv_bfloat16 h = __double2bfloat16(x);
-        hi[e] = h;
-        lo[e] = __double2bfloat16(x - (double)__bfloat162float(h));
-    } else {
-        __half h = __double2half(x);
-        hi[e] = h;
-        lo[e] = __double2half(x - (double)__half2float(h));
+    const int64_t r = blockIdx.x * 8LL + (threadIdx.x >> 5);
+    if (r >= rows) return;
+    const double* row = src + r * M;
+    uint32_t* oh = reinterpret_cast<uint32_t*>(hi + r * Mp);   // Mp is a multiple of 32
+    uint32_t* ol = reinterpret_cast<uint32_t*>(lo + r * Mp);
+    for (int J = 2 * (threadIdx.x & 31); J < Mp; J += 64) {
+        uint32_t h[2], l[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const double x = J + q < M ? row[J + q] : 0.0;
+            if constexpr (BF16) {
+                if (!split_bf16_bits(x, h[q], l[q])) {
+                    const __nv_bfloat16 t = __double2bfloat16(x);
+                    h[q] = __bfloat16_as_ushort(t);
+                    l[q] = __bfloat16_as_ushort(__double2bfloat16(x - (double)__bfloat162float(t)));
+                }
+            } else {
+                const __half t = __double2half(x * sc);
+                h[q] = __half_as_ushort(t);
+                l[q] = __half_as_ushort(__double2half(x * sc - (double)__half2float(t)));
+            }
+        }
+        oh[J >> 1] = h[0] | (h[1] << 16);
+        ol[J >> 1] = l[0] | (l[1] << 16);
     }
 }
+inline unsigned split16_grid(int64_t rows) { return (unsigned)((rows + 7) / 8); }
 
 // hi = tf32(x) (round to nearest on the 13 dropped bits), lo = fl32(x - hi);
 // the MMA reads lo's top 19 bits.  No scaling (FP32 exponent range); columns
@@ -842,13 +885,11 @@ static int split_all(const double* Lp, const double* Lov, int64_t rows_p, int64_
             CDS_LAUNCH_CHECK();
         }
     }
-    int64_t n1 = rows_p * Mp;
-    k_split16<T><<<(unsigned)((n1 + 255) / 256), 256, 0, stream>>>(
+    k_split16<T><<<split16_grid(rows_p), 256, 0, stream>>>(
         Lp, rows_p, M, Mp, lay.amax, (T*)lay.lp_hi, (T*)lay.lp_lo);
     CDS_LAUNCH_CHECK();
-    int64_t n2 = rows_ov * Mp;
-    if (n2 > 0) {
-        k_split16<T><<<(unsigned)((n2 + 255) / 256), 256, 0, stream>>>(
+    if (rows_ov > 0) {
+        k_split16<T><<<split16_grid(rows_ov), 256, 0, stream>>>(
             Lov, rows_ov, M, Mp, lay.amax + 1, (T*)lay.lov_hi, (T*)lay.lov_lo);
         CDS_LAUNCH_CHECK();
     }
@@ -890,7 +931,7 @@ size_t tc_cache_bytes(int32_t nmo, int32_t nocc, int32_t np) {
 
 namespace tc {
 template <int EC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 k_sigma_cached_grid(Params P, const float* __restrict__ cache, const float2* __restrict__ E2,
                     const float2* __restrict__ eps2, const int32_t* __restrict__ active,
                     double* __restrict__ part, int32_t nE, int32_t e_begin);
@@ -1068,6 +1109,29 @@ k_sigma_cached(Params P, const float* __restrict__ cache, const float2* __restri
     if (nslot > 0) flush();
 }
 
+// Two FP32 operations in one instruction (round to nearest in each half, as the
+// scalar operations).
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // Sigma and dSigma/dE of one work item at energies [e_begin, nE) of its
 // orbital from its cached numerators ct (the grid's energies past the ones
 // the tensor-core epilogue evaluates).  Thread = (row, column half) as in
@@ -1077,6 +1141,14 @@ k_sigma_cached(Params P, const float* __restrict__ cache, const float2* __restri
 // in a fixed order into out[e][2] (the partial row of the item, the layout
 // of k_sigma_tc), so the block meets at a barrier once per kRedE energies
 // instead of twice per pass.
+// The reciprocal (16 a clock and SM) is the bound, but with one instruction per
+// operation the issue slots (7 per element and energy, of the 8 clocks a
+// reciprocal takes a quarter of the SM) were nearly as tight: 24.4 ms for the
+// C60 shape's 20 orbitals x 63 energies against 17.6 ms of reciprocals.  Two
+// neighbouring columns share the packed operations here (5 slots); the sums
+// stay one column at a time, in the same order, so the results are the same bit
+// for bit (22.7 ms; the packed product alone or the scalar form measured no
+// faster, 23.7 and 24.5).  Columns of a ragged last block end at the next multiple of 16.
 // Et: the orbital's energies; ev: the molecule's orbital energies.
 template <int EC>
 __device__ __forceinline__ void cached_grid_item(const TermR& tm, int t, int s, int A, int B,
@@ -1087,7 +1159,8 @@ __device__ __forceinline__ void cached_grid_item(const TermR& tm, int t, int s, 
     constexpr int kRedE = 64;   // a multiple of every EC
     static_assert(kRedE % EC == 0, "energy chunk");
     __shared__ float red[8][kRedE][2];
-    __shared__ float2 sey[2][64];
+    // minus the columns' energies, pairs of columns: {-hi_j, -hi_j+1, -lo_j, -lo_j+1}
+    __shared__ float4 sey[2][32];
     (void)t;
     const int row = threadIdx.x & (TB - 1), half = threadIdx.x / TB;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1100,8 +1173,12 @@ __device__ __forceinline__ void cached_grid_item(const TermR& tm, int t, int s, 
 #pragma unroll
     for (int j = 0; j < 64; ++j) num[j] = (xok && j < ncols) ? ct[(int64_t)j * TB] : 0.f;
     // the previous item's reads of sey ended before its last flush's barriers
-    if (row < 64)      // padding columns: a far-off energy, so 0 * tiny
-        sey[half][row] = row < ncols ? ev[tm.eps_x_off + ybase + row] : make_float2(-1e30f, 0.f);
+    if (row < 64) {    // padding columns: a far-off energy, so 0 * tiny
+        const float2 e = row < ncols ? ev[tm.eps_x_off + ybase + row] : make_float2(-1e30f, 0.f);
+        float* d = reinterpret_cast<float*>(&sey[half][row >> 1]) + (row & 1);
+        d[0] = -e.x;
+        d[2] = -e.y;
+    }
     __syncthreads();
     float2 rb = make_float2(0.f, 0.f);
     if (xok) {
@@ -1111,26 +1188,35 @@ __device__ __forceinline__ void cached_grid_item(const TermR& tm, int t, int s, 
     }
     int fbase = e_begin;   // first energy of the chunk in red
     for (int e0 = e_begin; e0 < nE; e0 += EC) {
-        float ch[EC], cl[EC], as[EC], ad[EC];
+        float as[EC], ad[EC];
+        unsigned long long ch[EC], cl[EC];
 #pragma unroll
         for (int e = 0; e < EC; ++e) {
             const float2 c = df_add(Et[min(e0 + e, nE - 1)], rb);
-            ch[e] = c.x;
-            cl[e] = c.y;
+            ch[e] = pack2(c.x, c.x);
+            cl[e] = pack2(c.y, c.y);
             as[e] = 0.f;
             ad[e] = 0.f;
         }
         if (xok) {
 #pragma unroll
-            for (int j = 0; j < 64; ++j) {
-                const float2 e2 = sey[half][j];
+            for (int j0 = 0; j0 < 64; j0 += 16) {
+                if (j0 >= ncols) break;          // the same in the whole warp
 #pragma unroll
-                for (int e = 0; e < EC; ++e) {
-                    const float d = (ch[e] - e2.x) + (cl[e] - e2.y);
-                    const float r = rcp_approx(d);
-                    const float tt = num[j] * r;
-                    as[e] += tt;
-                    ad[e] = fmaf(-tt, r, ad[e]);
+                for (int j = j0; j < j0 + 16; j += 2) {
+                    const float4 e2 = sey[half][j >> 1];
+                    const unsigned long long eh = pack2(e2.x, e2.y), el = pack2(e2.z, e2.w);
+                    const unsigned long long nn = pack2(num[j], num[j + 1]);
+#pragma unroll
+                    for (int e = 0; e < EC; ++e) {
+                        const float2 d = unpack2(add2(add2(ch[e], eh), add2(cl[e], el)));
+                        const float r0 = rcp_approx(d.x), r1 = rcp_approx(d.y);
+                        const float2 tt = unpack2(mul2(nn, pack2(r0, r1)));
+                        as[e] += tt.x;
+                        ad[e] = fmaf(-tt.x, r0, ad[e]);
+                        as[e] += tt.y;
+                        ad[e] = fmaf(-tt.y, r1, ad[e]);
+                    }
                 }
             }
         }
@@ -1166,7 +1252,7 @@ __device__ __forceinline__ void cached_grid_item(const TermR& tm, int t, int s, 
 }
 
 template <int EC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 k_sigma_cached_grid(Params P, const float* __restrict__ cache, const float2* __restrict__ E2,
                     const float2* __restrict__ eps2, const int32_t* __restrict__ active,
                     double* __restrict__ part, int32_t nE, int32_t e_begin) {
@@ -1183,7 +1269,7 @@ k_sigma_cached_grid(Params P, const float* __restrict__ cache, const float2* __r
 
 // The same over a batch of molecules (the grid pass of tc_batch_pass).
 template <int EC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 k_sigma_cached_grid_batch(const MolDesc* __restrict__ mols, int32_t nmol, int64_t nitems,
                           const float* __restrict__ cache, const float2* __restrict__ E2,
                           const float2* __restrict__ eps2, double* __restrict__ part,
@@ -1315,16 +1401,16 @@ int mp2_tc(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double
     }
     // one array feeds both operands: one scale, inv = 1 / s^2
     CDS_CUDA_TRY(cudaMemsetAsync(lay.amax, 0, 2 * sizeof(unsigned long long), stream));
-    const int64_t rows = (int64_t)nocc * nv, n = rows * Mp;
+    const int64_t rows = (int64_t)nocc * nv;
     if (!bf16) {
         k_absmax<<<4 * 152, 256, 0, stream>>>(Lov, rows * M, lay.amax);
         CDS_LAUNCH_CHECK();
         CDS_CUDA_TRY(cudaMemcpyAsync(lay.amax + 1, lay.amax, sizeof(unsigned long long),
                                      cudaMemcpyDeviceToDevice, stream));
-        k_split16<__half><<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(
+        k_split16<__half><<<split16_grid(rows), 256, 0, stream>>>(
             Lov, rows, M, Mp, lay.amax, (__half*)lay.lov_hi, (__half*)lay.lov_lo);
     } else {
-        k_split16<__nv_bfloat16><<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(
+        k_split16<__nv_bfloat16><<<split16_grid(rows), 256, 0, stream>>>(
             Lov, rows, M, Mp, lay.amax, (__nv_bfloat16*)lay.lov_hi, (__nv_bfloat16*)lay.lov_lo);
     }
     CDS_LAUNCH_CHECK();
@@ -1620,19 +1706,19 @@ int tc_batch_split(int32_t nmol, const BatchMol* mols, const int32_t* M, const B
         }
         if (rp) {
             if (bf16)
-                k_split16<__nv_bfloat16><<<(unsigned)((rp * Mp + 255) / 256), 256, 0, stream>>>(
+                k_split16<__nv_bfloat16><<<split16_grid(rp), 256, 0, stream>>>(
                     lp, rp, M[c], Mp, lay.amax + 2 * c, (__nv_bfloat16*)lp_hi, (__nv_bfloat16*)lp_lo);
             else
-                k_split16<__half><<<(unsigned)((rp * Mp + 255) / 256), 256, 0, stream>>>(
+                k_split16<__half><<<split16_grid(rp), 256, 0, stream>>>(
                     lp, rp, M[c], Mp, lay.amax + 2 * c, (__half*)lp_hi, (__half*)lp_lo);
             CDS_LAUNCH_CHECK();
         }
         if (ro) {
             if (bf16)
-                k_split16<__nv_bfloat16><<<(unsigned)((ro * Mp + 255) / 256), 256, 0, stream>>>(
+                k_split16<__nv_bfloat16><<<split16_grid(ro), 256, 0, stream>>>(
                     lov, ro, M[c], Mp, lay.amax + 2 * c + 1, (__nv_bfloat16*)ov_hi, (__nv_bfloat16*)ov_lo);
             else
-                k_split16<__half><<<(unsigned)((ro * Mp + 255) / 256), 256, 0, stream>>>(
+                k_split16<__half><<<split16_grid(ro), 256, 0, stream>>>(
                     lov, ro, M[c], Mp, lay.amax + 2 * c + 1, (__half*)ov_hi, (__half*)ov_lo);
             CDS_LAUNCH_CHECK();
         }
