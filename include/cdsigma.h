@@ -203,8 +203,10 @@ int cds_cd_live_pairs(int32_t nbf, const void* workspace, int32_t precision, int
 int cds_cd_candidates(int32_t precision);
 
 /* Workspace of cds_cd_decompose for one precision and max_rank (OZAKI holds a
- * slice store of max_rank columns; cds_cd_workspace_bytes covers FP64 and
- * F32X2 for any max_rank). */
+ * slice store of max_rank columns, FP64 of up to 768 pairs per SM its rows as
+ * integers, 8 bytes each, for the form that runs as one launch;
+ * cds_cd_workspace_bytes covers FP64, a launch per step, and F32X2 for any
+ * max_rank). */
 size_t cds_cd_workspace_bytes_prec(int32_t nbf, int32_t max_rank, int32_t precision);
 
 /* Kernel timing of the OZAKI decomposition's projection GEMM (the tcgen05
@@ -581,11 +583,13 @@ typedef struct {
 int cds_batch_offsets(int32_t nmol, const cds_mol* mols, int64_t* offs);
 
 /* Host only.  precision CDS_PREC_OZAKI adds the region of the batched
- * tensor-core decomposition after the worker slots; any other value leaves
- * it out.  The calls accept a workspace without the slots (the scratch and
+ * tensor-core decomposition after the worker slots, CDS_PREC_FP64 that of the
+ * FP64 decomposition in one launch per group of molecules; any other value
+ * leaves them out.  The calls accept a workspace without the slots (the scratch and
  * state parts only); the transform then runs the molecules one after the
  * other on the caller's stream, and the tensor-core decomposition returns
- * CDS_ERR_WORKSPACE. */
+ * CDS_ERR_WORKSPACE.  Without its region the FP64 decomposition takes a
+ * launch per step. */
 size_t cds_batch_workspace_bytes(int32_t nmol, const cds_mol* mols, int32_t precision);
 
 /* Blocking.  Per molecule as cds_cd_decompose (delta and scheme shared);

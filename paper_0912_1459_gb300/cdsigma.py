@@ -714,9 +714,8 @@ class Batch:
         self.total = self.off[self.n]
         self.prec = precision
         need = self.lib.cds_batch_workspace_bytes(self.n, self.mols, PRECISIONS[precision])
-        if cd_precision == "ozaki":
-            need = max(need, self.lib.cds_batch_workspace_bytes(self.n, self.mols,
-                                                                PRECISIONS["ozaki"]))
+        own = "ozaki" if cd_precision == "ozaki" else "fp64"   # the decomposition's own region
+        need = max(need, self.lib.cds_batch_workspace_bytes(self.n, self.mols, PRECISIONS[own]))
         self.ws = _workspace(need, self.dev)
         f64 = dict(dtype=torch.float64, device=self.dev)
         i32 = dict(dtype=torch.int32, device=self.dev)

@@ -32,7 +32,8 @@ size_t cd_batch_workspace_bytes(int32_t nmol, const BatchMol* mols);
 int cd_batch_decompose(int32_t nmol, const BatchMol* mols, const BatchOffsets* off,
                        const double* xyz, const double* alpha, const int32_t* atom, double delta,
                        int32_t scheme, int32_t precision, double* L, int32_t* piv, double* D,
-                       int32_t* M_out, void* ws, size_t ws_bytes, cudaStream_t stream);
+                       int32_t* M_out, void* ws, size_t ws_bytes, void* direct, cudaStream_t stream);
+size_t cd_batch_direct_bytes(int32_t nmol, const BatchMol* mols);
 size_t cd_tc_batch_workspace_bytes(int32_t nmol, const BatchMol* mols);
 int cd_batch_decompose_tc(int32_t nmol, const BatchMol* mols, const BatchOffsets* off,
                           const double* xyz, const double* alpha, const int32_t* atom,
@@ -370,17 +371,19 @@ static size_t base_bytes(int32_t nmol, const cds_mol* mols) {
            align_up(qp_batch_layout(nullptr, nmol, bm.data(), tot.orb).bytes);
 }
 
-// The tensor-core decomposition's region (CDS_PREC_OZAKI) follows the slots.
-static size_t tc_cd_bytes(int32_t nmol, const cds_mol* mols, int32_t precision) {
-    if (precision != CDS_PREC_OZAKI) return 0;
+// The tensor-core decomposition's region (CDS_PREC_OZAKI), or the one-launch FP64
+// form's (CDS_PREC_FP64), follows the slots.
+static size_t cd_region_bytes(int32_t nmol, const cds_mol* mols, int32_t precision) {
+    if (precision != CDS_PREC_OZAKI && precision != CDS_PREC_FP64) return 0;
     std::vector<BatchMol> bm = to_internal(nmol, mols);
+    if (precision == CDS_PREC_FP64) return cd_batch_direct_bytes(nmol, bm.data());
     return cd_tc_batch_workspace_bytes(nmol, bm.data());
 }
 
 extern "C" size_t cds_batch_workspace_bytes(int32_t nmol, const cds_mol* mols, int32_t precision) {
     if (!mols_ok(nmol, mols)) return 0;
     return base_bytes(nmol, mols) + kWorkers * worker_slot_bytes(nmol, mols) +
-           tc_cd_bytes(nmol, mols, precision);
+           cd_region_bytes(nmol, mols, precision);
 }
 
 // The worker slots of a workspace of `bytes` bytes, or null when it has none.
@@ -411,7 +414,7 @@ extern "C" int cds_batch_cd_decompose(int32_t nmol, const cds_mol* mols, const d
         return CDS_ERR_ARG;
     if (precision == CDS_PREC_OZAKI) {
         const size_t before = base_bytes(nmol, mols) + kWorkers * worker_slot_bytes(nmol, mols);
-        const size_t need = tc_cd_bytes(nmol, mols, precision);
+        const size_t need = cd_region_bytes(nmol, mols, precision);
         if (!workspace || workspace_bytes < before + need) return CDS_ERR_WORKSPACE;
         std::vector<BatchMol> bm = to_internal(nmol, mols);
         std::vector<BatchOffsets> off = offsets_of(nmol, mols, nullptr);
@@ -422,9 +425,15 @@ extern "C" int cds_batch_cd_decompose(int32_t nmol, const cds_mol* mols, const d
     if (workspace_bytes < base_bytes(nmol, mols)) return CDS_ERR_WORKSPACE;
     std::vector<BatchMol> bm = to_internal(nmol, mols);
     std::vector<BatchOffsets> off = offsets_of(nmol, mols, nullptr);
+    // a caller's workspace may lack the slots, or the region behind them
+    const size_t before = base_bytes(nmol, mols) + kWorkers * worker_slot_bytes(nmol, mols);
+    const size_t region = precision == CDS_PREC_FP64 ? cd_region_bytes(nmol, mols, precision) : 0;
+    void* direct = workspace && region && workspace_bytes >= before + region
+                       ? static_cast<char*>(workspace) + before
+                       : nullptr;
     return cd_batch_decompose(nmol, bm.data(), off.data(), xyz, alpha, atom, delta, scheme,
                               precision, L, piv, D, M_out, workspace,
-                              cd_batch_workspace_bytes(nmol, bm.data()), stream);
+                              cd_batch_workspace_bytes(nmol, bm.data()), direct, stream);
 }
 
 extern "C" int cds_batch_cd_to_mo(int32_t nmol, const cds_mol* mols, const int32_t* M,

@@ -81,13 +81,16 @@ __device__ __forceinline__ bool eri_is_far(double x, double s) { return x >= kEr
 __device__ __forceinline__ double eri_far(double kk, double x) { return kPi3 * kk * rsqrt(x); }
 // T < kErfOneT: F0(T) from its Taylor expansion around the nearest point of a
 // 1/16 grid (boys_table.h: F_0(T_i + d) = sum_m F_m(T_i) (-d)^m / m!, eight
-// terms, truncation below 2e-18).  kk = (K_I/p)(K_J/q).
-__device__ __forceinline__ double eri_near(double kk, double x, double s) {
+// terms, truncation below 2e-18).  kk = (K_I/p)(K_J/q).  BS: row stride of the
+// table at boys (the global one, or a caller's copy in shared memory).
+template <int BS = kBoysOrder>
+__device__ __forceinline__ double eri_near(double kk, double x, double s,
+                                           const double* boys = &kBoysTaylor[0][0]) {
     const double rs = rsqrt(s);
     const double T = x * (rs * rs);
     const int i = min(max(__double2int_rn(T * kBoysPerUnit), 0), kBoysPoints - 1);
     const double d = T - (double)i * (1.0 / kBoysPerUnit);
-    const double* c = kBoysTaylor[i];
+    const double* c = boys + i * BS;
     double f = c[kBoysOrder - 1];
 #pragma unroll
     for (int m = kBoysOrder - 2; m >= 0; --m) f = fma(f, d, c[m]);
