@@ -16,10 +16,12 @@
 // bits).  x = sigma (sum_s slice_s + O(2^-42)).
 // Products: slice pairs (s, t) with s + t <= 7 (21 pairs; the dropped ones
 // are below 2^-49).  For one pair sum_k |d_s e_t| <= K 127^2 < 2^24 when
-// K <= 1040, so each of the six leading pairs (s + t <= 4) accumulates
-// exactly in its own FP32 TMEM accumulator; the 15 others share a seventh,
-// whose rounding is below 2^-45 of sigma_A sigma_B K.  The epilogue adds the
-// seven in float-pair arithmetic and scales by sigma_A sigma_B.
+// K <= 1040, so the leading pairs accumulate exactly in FP32: the pair with
+// s + t = 2 and the two with s + t = 3 each in its own TMEM accumulator, the
+// three with s + t = 4 together in one that is emptied (to integers) every 320
+// k, 3 x 320 x 127^2 < 2^24.  The 15 others share a fifth, whose rounding is
+// below 2^-45 of sigma_A sigma_B K.  The epilogue adds all in float-pair
+// arithmetic and scales by sigma_A sigma_B.
 //
 // Per batch of kb vectors, as in the split-precision form:
 //   GEMM 1   T^T[(K, nu)][r] = sum_mu A^K[nu][mu] Cj[mu][r]   -> T as float pairs
@@ -27,12 +29,19 @@
 //   GEMM 3   Lp[t][q][K]     = sum_nu T[(o + t, K)][nu] C[nu][q]
 // with every operand sliced by rows (U rows (K, nu), Cj / C columns, T rows).
 //
-// Kernel: M tile 128, N tile 64, tiles ordered N fastest (the CTAs that share
-// an A tile run together, so it is read from DRAM once); 3 TMA stages of
-// {6 A slices, 6 B slices}
-// (64-byte swizzled rows of 32 BF16); warp 0 = TMA producer, warp 1 = TMEM
-// allocator + MMA issuer (21 MMAs per 16 k), warps 2..5 = epilogue.  Every
-// wait is bounded and sets an error word instead of hanging.
+// Kernel: M tile 128, N tile tn <= 96 (multiple of 16), tiles ordered N fastest
+// (the CTAs that share an A tile run together, so it is read from DRAM once); 2 TMA
+// stages of {6 A slices, 6 B slices} (64-byte swizzled rows of 32 BF16); warp 0 = TMA
+// producer, warp 1 = TMEM allocator + MMA issuer (21 MMAs per 16 k), warps 2..9 =
+// epilogue.  Every wait is bounded and sets an error word instead of hanging.
+//
+// What bounds it: an MMA reads its operands from shared memory at 128 bytes a clock,
+// (4 KB + 32 N) / 128 clocks against 32 N / 64 of arithmetic, i.e. 48 clocks at N = 64
+// (67 % of the peak), 56 at 96 (86 %), 64 at 128, and the TMA's writes share that
+// port.  With one accumulator per leading pair (seven, N = 64) and the outputs converted
+// to FP64 (2 conversions a clock and SM) before TMEM was free for the next tile, the
+// transform of 896 vectors of 840 functions took 18.9 ms; with five, N = 96 and TMEM
+// freed first, 15.8 (5 ms of it the slicing).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -49,41 +58,44 @@ using namespace tc;
 constexpr int S = 6;                             // slices per operand
 constexpr int BETA = 7;                          // bits per slice
 constexpr int QBITS = S * BETA;                  // 42-bit fixed point
-constexpr int NACC = 7;                          // TMEM accumulators
+constexpr int NACC = 5;                          // TMEM accumulators
+constexpr int ACC_MID = 3;                       // the one of the pairs s + t = 4
+constexpr int MID_KB = 10;                       // k-blocks after which it is emptied
 constexpr int TM = 128;
-constexpr int TN = 64;
+constexpr int TN = 96;                           // widest N tile
 constexpr int KE = 32;                           // BF16 per k-block (64-byte rows)
-constexpr int NSTAGE = 3;
+constexpr int NSTAGE = 2;
 constexpr int A_SLICE = TM * 64;                 // 8 KB
-constexpr int B_SLICE = TN * 64;                 // 4 KB
-constexpr int STAGE_BYTES = S * (A_SLICE + B_SLICE);   // 72 KB
-constexpr int EPI_WARPS = 4;
+constexpr int B_SLICE = TN * 64;                 // 6 KB
+constexpr int STAGE_BYTES = S * (A_SLICE + B_SLICE);   // 84 KB
+constexpr int EPI_WARPS = 8;                     // two per TMEM lane quarter, half the columns each
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
-constexpr uint32_t TMEM_COLS = 512;              // 7 x 64 used
+constexpr uint32_t TMEM_COLS = 512;              // 5 x 96 used
 constexpr size_t SMEM_BYTES = 1024 + NSTAGE * STAGE_BYTES + 256;
 constexpr int MAX_K = 1040;                      // exact accumulation bound (K 127^2 < 2^24)
 
-// kind::f16 descriptor: D f32, A/B bf16, K-major, N = 64, M = 128
-constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                        ((uint32_t)(TM >> 4) << 24);
+static_assert(3 * MID_KB * KE * 127 * 127 < (1 << 24), "exact sums in FP32");
 
-// (s, t) slice pairs with s + t <= 7 (0-based u = s + t <= 5), leading
-// first; accumulators 0..5 take the pairs with u <= 2 one each, 6 the rest;
-// first = the pair is the first one issued into its accumulator.
+// kind::f16 descriptor without N: D f32, A/B bf16, K-major, M = 128
+constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
+
+// (s, t) slice pairs with s + t <= 7 (0-based u = s + t <= 5) in the order of issue:
+// u = 0, u = 1, u >= 3, then u = 2, whose accumulator may still have to be emptied.
 constexpr int NPAIRS = 21;
+constexpr int NMID = 3;
 struct PairTab {
-    int s[NPAIRS], t[NPAIRS], acc[NPAIRS], first[NPAIRS];
+    int s[NPAIRS], t[NPAIRS], acc[NPAIRS], first[NPAIRS];   // first: into its accumulator
 };
 __host__ __device__ constexpr PairTab make_pairs() {
     PairTab p{};
     bool seen[NACC] = {};
     int n = 0;
-    for (int u = 0; u <= S - 1; ++u)
-        for (int s = 0; s <= u; ++s) {
-            const int t = u - s;
-            const int acc = u == 0 ? 0 : u == 1 ? 1 + s : u == 2 ? 3 + s : 6;
+    const int order[S] = {0, 1, 3, 4, 5, 2};
+    for (int i = 0; i < S; ++i)
+        for (int s = 0; s <= order[i]; ++s) {
+            const int u = order[i], acc = u == 0 ? 0 : u == 1 ? 1 + s : u == 2 ? ACC_MID : 4;
             p.s[n] = s;
-            p.t[n] = t;
+            p.t[n] = u - s;
             p.acc[n] = acc;
             p.first[n] = seen[acc] ? 0 : 1;
             seen[acc] = true;
@@ -91,14 +103,15 @@ __host__ __device__ constexpr PairTab make_pairs() {
         }
     return p;
 }
-static_assert(make_pairs().acc[NPAIRS - 1] == 6 && make_pairs().s[NPAIRS - 1] == 5, "pair table");
+static_assert(make_pairs().acc[NPAIRS - NMID] == ACC_MID && make_pairs().acc[NPAIRS - NMID - 1] == 4,
+              "pair table");
 
 struct Maps {
     CUtensorMap a, b;   // 3-D {k, rows, slice}
 };
 
 struct Args {
-    int32_t m, n, kblocks, mtiles, ntiles;
+    int32_t m, n, tn, kblocks, mtiles, ntiles;
     const float* sa;   // row scales of A (powers of two)
     const float* sb;   // row scales of B
     // output element (row m, column c) at (m / kdiv) rs_hi + (m % kdiv) rs_lo + c cs
@@ -125,7 +138,7 @@ __device__ __forceinline__ bool epi_any(bool v) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, 128, p;\n\t"
+        "bar.red.or.pred q, 1, 256, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
         : "r"((uint32_t)v)
@@ -143,7 +156,9 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
     uint64_t* empty = bars + NSTAGE;
     uint64_t* tfull = bars + 2 * NSTAGE;
     uint64_t* tempty = tfull + 1;
-    uint32_t* tmem_slot = (uint32_t*)(tempty + 1);
+    uint64_t* mfull = tempty + 1;      // accumulator ACC_MID full / emptied between its chunks
+    uint64_t* mempty = mfull + 1;
+    uint32_t* tmem_slot = (uint32_t*)(mempty + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = (int64_t)g.mtiles * g.ntiles;
@@ -153,6 +168,8 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
         for (int i = 0; i < NSTAGE; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
         mbar_init(tfull, 1);
         mbar_init(tempty, EPI_WARPS);
+        mbar_init(mfull, 1);
+        mbar_init(mempty, EPI_WARPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -171,6 +188,7 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
             // ---------------- TMA producer ----------------
             int stage = 0;
             uint32_t phase = 0;
+            const uint32_t bytes = S * (A_SLICE + 64u * (uint32_t)g.tn);
             int32_t last_parity[NSTAGE];
             for (int i = 0; i < NSTAGE; ++i) last_parity[i] = -1;
             bool ok = true;
@@ -178,13 +196,13 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
                 const int nt = (int)(tile % g.ntiles), mt = (int)(tile / g.ntiles);
                 for (int kb = 0; kb < g.kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, verr)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&full[stage], (uint32_t)STAGE_BYTES);
+                    mbar_arrive_expect_tx(&full[stage], bytes);
                     last_parity[stage] = (int32_t)phase;
                     const uint32_t st = smem_u32(stages + stage * STAGE_BYTES);
                     for (int s = 0; s < S; ++s) {
                         tma_load_3d(st + s * A_SLICE, &maps.a, &full[stage], kb * KE, mt * TM, s);
                         tma_load_3d(st + S * A_SLICE + s * B_SLICE, &maps.b, &full[stage], kb * KE,
-                                    nt * TN, s);
+                                    nt * g.tn, s);
                     }
                     if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
                 }
@@ -196,8 +214,9 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
             constexpr PairTab kPairs = make_pairs();
+            const uint32_t id = ID | ((uint32_t)(g.tn >> 3) << 17);
             int stage = 0;
-            uint32_t phase = 0, aphase = 0;
+            uint32_t phase = 0, aphase = 0, mphase = 0;
             bool ok = true;
             for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
                 if (!mbar_wait(tempty, aphase ^ 1u, verr)) break;
@@ -206,18 +225,29 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
                     if (!mbar_wait(&full[stage], phase, verr)) { ok = false; break; }
                     fence_after();
                     const uint32_t base = smem_u32(stages + stage * STAGE_BYTES);
-#pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {   // 16 BF16 (32 bytes) of k per MMA
+                    auto issue = [&](int p, int kk, bool fresh) {   // 16 BF16 (32 bytes) of k
                         const uint32_t off = kk * 32;
+                        mma_f16(tmem + (uint32_t)kPairs.acc[p] * TN,
+                                sdesc(base + kPairs.s[p] * A_SLICE + off),
+                                sdesc(base + S * A_SLICE + kPairs.t[p] * B_SLICE + off), id,
+                                (fresh && kk == 0 && kPairs.first[p]) ? 0u : 1u);
+                    };
 #pragma unroll
-                        for (int p = 0; p < NPAIRS; ++p) {
-                            const uint32_t en = ((kb | kk) || !kPairs.first[p]) ? 1u : 0u;
-                            mma_f16(tmem + (uint32_t)kPairs.acc[p] * TN,
-                                    sdesc(base + kPairs.s[p] * A_SLICE + off),
-                                    sdesc(base + S * A_SLICE + kPairs.t[p] * B_SLICE + off), ID, en);
-                        }
+                    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                        for (int p = 0; p < NPAIRS - NMID; ++p) issue(p, kk, kb == 0);
+                    const bool again = kb > 0 && kb % MID_KB == 0;   // a new chunk: emptied meanwhile
+                    if (again) {
+                        if (!mbar_wait(mempty, mphase, verr)) { ok = false; break; }
+                        mphase ^= 1u;
+                        fence_after();
                     }
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                        for (int p = NPAIRS - NMID; p < NPAIRS; ++p) issue(p, kk, kb % MID_KB == 0);
                     mma_commit(&empty[stage]);
+                    if ((kb + 1) % MID_KB == 0 && kb + 1 < g.kblocks) mma_commit(mfull);
                     if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
@@ -226,44 +256,62 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
             }
         }
     } else {
-        // ---------------- epilogue (4 warps, one output row per thread) ----------------
-        const int quad = warp & 3;
+        // ---------------- epilogue (one output row and half the columns per thread) ----------------
+        const int quad = warp & 3, half = (warp - 2) >> 2;
         const int row = quad * 32 + lane;
-        uint32_t aphase = 0;
+        const int hw = g.tn / 2;                    // columns of this warp, a multiple of 8
+        constexpr int C8 = TN / 2 / 8;
+        constexpr float MID_UP = 268435456.f, MID_DOWN = 1.f / 268435456.f;   // 2^28
+        uint32_t aphase = 0, mphase = 0;
         for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-            const bool bad = !mbar_wait(tfull, aphase, verr) || *verr;
+            const int nt = (int)(tile % g.ntiles), mt = (int)(tile / g.ntiles);
+            const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * hw);
+            int mid[C8][8];
+#pragma unroll
+            for (int c = 0; c < C8; ++c)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) mid[c][j] = 0;
+            bool bad = false;
+            for (int kb = MID_KB; kb < g.kblocks && !bad; kb += MID_KB) {   // chunks but the last
+                bad = !mbar_wait(mfull, mphase, verr);
+                mphase ^= 1u;
+                if (bad) break;
+                fence_after();
+#pragma unroll
+                for (int c = 0; c < C8; ++c) {
+                    if (8 * c < hw) {
+                        float a[8];
+                        tmem_ld8(ta + (uint32_t)(ACC_MID * TN + 8 * c), a);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) mid[c][j] += __float2int_rn(a[j] * MID_UP);
+                    }
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(mempty);
+            }
+            bad = bad || !mbar_wait(tfull, aphase, verr) || *verr;
             if (epi_any(bad)) break;
             fence_after();
-            const int nt = (int)(tile % g.ntiles), mt = (int)(tile / g.ntiles);
-            const int64_t m = (int64_t)mt * TM + row;
-            const bool mok = m < g.m;
-            const int64_t ob = mok ? (m / g.kdiv) * g.rs_hi + (m % g.kdiv) * g.rs_lo : 0;
-            const float sa = mok ? g.sa[m] : 0.f;
-            const int c_base = nt * TN;
-            const int ncols = min(TN, g.n - c_base);
-            const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16);
-            if ((int64_t)mt * TM + quad * 32 < g.m) {
-#pragma unroll 1
-                for (int c0 = 0; c0 < ncols; c0 += 16) {
-                    float a[NACC][16];
+            float2 v[C8][8];
 #pragma unroll
-                    for (int q = 0; q < NACC; ++q) tmem_ld16(ta + (uint32_t)q * TN + c0, a[q]);
+            for (int c = 0; c < C8; ++c) {
+                if (8 * c < hw) {
+                    float a[NACC][8];
+#pragma unroll
+                    for (int q = 0; q < NACC; ++q) tmem_ld8(ta + (uint32_t)(q * TN + 8 * c), a[q]);
                     tmem_wait_ld();
-                    if (mok) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int c = c_base + c0 + j;
-                            if (c0 + j < ncols) {
-                                // smallest first: rest, then the exact leading pairs
-                                float2 v = make_float2(a[6][j], 0.f);
-#pragma unroll
-                                for (int q = 5; q >= 0; --q) v = pair_add(v, a[q][j]);
-                                const float st = sa * g.sb[c];   // power of two
-                                const int64_t e = ob + (int64_t)c * g.cs;
-                                if (g.out) g.out[e] = (double)(v.x * st) + (double)(v.y * st);
-                                else g.outf[e] = make_float2(v.x * st, v.y * st);
-                            }
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        // smallest first: the rest, then the exact leading sums
+                        const int u = mid[c][j] + __float2int_rn(a[ACC_MID][j] * MID_UP);   // below 2^26
+                        float2 x = make_float2(a[4][j], 0.f);
+                        x = pair_add(x, (float)(u & 4095) * MID_DOWN);
+                        x = pair_add(x, (float)(u & ~4095) * MID_DOWN);
+                        x = pair_add(x, a[2][j]);
+                        x = pair_add(x, a[1][j]);
+                        v[c][j] = pair_add(x, a[0][j]);
                     }
                 }
             }
@@ -271,6 +319,25 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty);
             aphase ^= 1u;
+            // the next tile's products go on meanwhile
+            const int64_t m = (int64_t)mt * TM + row;
+            if (m < g.m) {
+                const int64_t ob = (m / g.kdiv) * g.rs_hi + (m % g.kdiv) * g.rs_lo;
+                const float sa = g.sa[m];
+                const int c_base = nt * g.tn + half * hw;
+#pragma unroll
+                for (int c = 0; c < C8; ++c)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int col = c_base + 8 * c + j;
+                        if (8 * c < hw && col < g.n) {
+                            const float st = sa * g.sb[col];   // power of two
+                            const int64_t e = ob + (int64_t)col * g.cs;
+                            if (g.out) g.out[e] = (double)(v[c][j].x * st) + (double)(v[c][j].y * st);
+                            else g.outf[e] = make_float2(v[c][j].x * st, v[c][j].y * st);
+                        }
+                    }
+            }
         }
     }
 
@@ -545,7 +612,9 @@ int run_gemm(const __nv_bfloat16* a, int64_t a_plane, const float* sa, int64_t a
     g.n = (int32_t)b_rows;
     g.kblocks = (kdim + KE - 1) / KE;
     g.mtiles = (g.m + TM - 1) / TM;
-    g.ntiles = (g.n + TN - 1) / TN;
+    const int32_t nt = (g.n + TN - 1) / TN;   // the fewest tiles, of even width
+    g.tn = ((g.n + nt - 1) / nt + 15) / 16 * 16;
+    g.ntiles = (g.n + g.tn - 1) / g.tn;
     g.sa = sa;
     g.sb = sb;
     g.kdiv = kdiv;
@@ -556,7 +625,7 @@ int run_gemm(const __nv_bfloat16* a, int64_t a_plane, const float* sa, int64_t a
     g.outf = outf;
     Maps maps;
     if (!make_slice_map(&maps.a, a, kdim, a_rows, ld, a_plane, TM) ||
-        !make_slice_map(&maps.b, b, kdim, b_rows, ld, b_plane, TN))
+        !make_slice_map(&maps.b, b, kdim, b_rows, ld, b_plane, (uint32_t)g.tn))
         return CDS_ERR_CUDA;
     // per launch: the attribute belongs to the current device
     CDS_CUDA_TRY(cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
