@@ -145,12 +145,11 @@ __device__ __forceinline__ double warp_sums4(const double (&v)[4]) {
 }
 
 // 32 x 32 tiles (x, c2) of up to kC1 values of c1 in turn: G in both layouts, the
-// energy partials and dSigma/dw of orbital t.  The FP64 pipe bounds it: about 11
-// operations per element here (8 for D, its reciprocal, G and r, 2.4 for the sums
+// energy partials and dSigma/dw of orbital t.  The FP64 pipe bounds it: about 10
+// operations per element here (7 for D, its reciprocal, G and r, 2.4 for the sums
 // over x, c2 and c1, which meet across the warp once per kC1 tiles), 60 with
 // divisions, a warp sum per row and the splits' conversions on that pipe too
-// (60.6 ms of an
-// 80.2 ms gradient of 8 orbitals of 840 functions; 39.7 ms in all now).
+// (60.6 ms of an 80.2 ms gradient of 8 orbitals of 840 functions; 18.4 of 32.7 now).
 constexpr int kC1 = 4;
 template <bool TF32>
 __global__ void __launch_bounds__(256)
@@ -206,21 +205,23 @@ k_adj_gx(GxArgs a, int32_t t, int32_t nmo, const double* __restrict__ eps,
             const int32_t x = x0 + i;
             const bool ok = x < a.nx && cok;
             const double p = a.swap_c1 ? yx[q] : sP[i][tx];
-            double G = 0.0, r = 0.0;
+            double r = 0.0;
             if (ok) {
                 const double rc = recip(sa[i] + bt);
                 const double n = fma(2.0, y[q], -p);   // 2 X - X_partner
                 const double h = n * rc;
-                G = 2.0 * h;
                 r = h * (y[q] * rc);
                 uint32_t pk;
-                if constexpr (TF32) {
-                    split_d<TF32>(G, &sH[i][tx], &sL[i][tx], 0);
-                } else if (split_bits(G, pk)) {
-                    sH[i][tx] = (uint16_t)pk;
-                    sL[i][tx] = (uint16_t)(pk >> 16);
+                // G = 2 h: by its exponent where split_bits takes it (zero, infinity and NaN
+                // wrap out of its range), as the FP64 units bound this kernel
+                bool split = false;
+                if constexpr (!TF32)
+                    split = split_bits(__longlong_as_double(__double_as_longlong(h) + (1ll << 52)), pk);
+                if (split) {
+                    sH[i][tx] = (E<TF32>)(uint16_t)pk;
+                    sL[i][tx] = (E<TF32>)(uint16_t)(pk >> 16);
                 } else {
-                    split_d<TF32>(G, &sH[i][tx], &sL[i][tx], 0);
+                    split_d<TF32>(2.0 * h, &sH[i][tx], &sL[i][tx], 0);
                 }
                 const int64_t e = ((int64_t)a.tl * a.nx + x) * a.ldc + col0 + c2_0 + tx;
                 gah[e] = sH[i][tx];
@@ -361,10 +362,12 @@ int gradient(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const doub
             for (int sum = 0; sum < 2; ++sum) {
                 const int32_t nx = sum == 0 ? o : v, xoff = sum == 0 ? 0 : o;
                 const size_t arow = ((size_t)tl * nmo + xoff) * l.ldM * sizeof(T);
-                // X[x][c] = sum_J Lq[x][J] Lov[c][J]
-                int st = tr_split_gemm(precision, (char*)l.lq_hi + arow, (char*)l.lq_lo + arow, nx,
-                                       l.lov_hi, l.lov_lo, ov, M, l.ldM, nx, 0, l.ldc, 1, l.X,
-                                       false, l.err, stream);
+                // X[x][c] = sum_J Lq[x][J] Lov[c][J], the rows c as the products' rows: a
+                // warp then stores 32 consecutive c, and not to 32 rows a megabyte apart
+                // (180 x 118,800, M = 896: 0.29 -> 0.23 ms)
+                int st = tr_split_gemm(precision, l.lov_hi, l.lov_lo, ov, (char*)l.lq_hi + arow,
+                                       (char*)l.lq_lo + arow, nx, M, l.ldM, ov, 0, 1, l.ldc, l.X,
+                                       false, l.err, stream, true);
                 if (st) return st;
                 GxArgs a;
                 a.X = l.X;

@@ -19,13 +19,21 @@
 // Both need no scaling (FP32 exponent range).
 //
 // One kernel serves the three GEMMs: D[m][n] = sum_k A[m][k] B[n][k], both
-// operands K-major (k contiguous), M tile 128, N tile tn <= 128 (multiple of
-// 16), a persistent grid walking the tiles.  Warp 0 = TMA producer, warp 1 =
-// TMEM allocator + MMA issuer, warps 2..5 = epilogue (one output row per
+// operands K-major (k contiguous), a persistent grid walking the tiles of 128 x tn
+// (tn <= 128, a multiple of 16), or, once there are enough tiles for every pair of
+// SMs, of 256 x tn (a multiple of 32) by two CTAs each, which halves what B takes of
+// the shared memory's and the L2's bandwidth.  Warp 0 = TMA producer, warp 1 =
+// TMEM allocator + MMA issuer, warps 2..9 = epilogue (half an output row per
 // thread).  Shared memory holds NSTAGE stages of {A_hi, A_lo, B_hi, B_lo}
 // (rows of 64 bytes, 64-byte swizzle); TMEM holds two accumulator pairs so
 // the epilogue of one tile overlaps the MMAs of the next.  Every wait is
 // bounded (2 s of %globaltimer) and sets an error word instead of hanging.
+//
+// What bounds it: with few k the epilogue, until its conversions to FP64 (one a clock
+// and SM) became integer operations, 660 x 118,800 outputs of K = 896 0.81 -> 0.46 ms;
+// with many k the operands' delivery, 5,280 x 896 of K = 118,800 2.6 ms (1.3 PFLOP/s).
+// Walking the side with fewer tiles first reads the larger operand from DRAM once:
+// 118,800 x 896 of K = 5,280 3.2 -> 2.6 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -49,7 +57,7 @@ constexpr int NSTAGE = 4;
 constexpr int A_TILE = TM * ROW_BYTES;          // 8 KB
 constexpr int B_TILE = 128 * ROW_BYTES;         // 8 KB (tn <= 128 rows)
 constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;
-constexpr int EPI_WARPS = 4;
+constexpr int EPI_WARPS = 8;                     // two per TMEM lane quarter
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr uint32_t TMEM_COLS = 512;             // 2 buffers x (hi.hi + cross) x 128
 constexpr size_t SMEM_BYTES = 1024 + NSTAGE * STAGE_BYTES + 256;
@@ -76,15 +84,25 @@ struct Args {
     void* out_hi;  // split output (operand containers)
     void* out_lo;
     int32_t accumulate;   // FP64 output: add to it instead of overwriting
+    int32_t lo_first;     // lo.hi before hi.lo: the sums of the call with A and B exchanged
 };
 
-// Barrier over the 128 epilogue threads that ORs a flag across them.
+// Tiles in the order of the side that has fewer of them: the CTAs at work share the
+// tiles of the larger operand, which is then read from DRAM once.
+__device__ __forceinline__ int tile_m(const Args& g, int64_t tile) {
+    return (int)(g.ntiles < g.mtiles ? tile / g.ntiles : tile % g.mtiles);
+}
+__device__ __forceinline__ int tile_n_of(const Args& g, int64_t tile) {
+    return (int)(g.ntiles < g.mtiles ? tile % g.ntiles : tile / g.mtiles);
+}
+
+// Barrier over the 256 epilogue threads that ORs a flag across them.
 __device__ __forceinline__ bool epi_any(bool v) {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, 128, p;\n\t"
+        "bar.red.or.pred q, 1, 256, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
         : "r"((uint32_t)v)
@@ -92,7 +110,19 @@ __device__ __forceinline__ bool epi_any(bool v) {
     return r != 0;
 }
 
-template <bool TF32>
+__device__ __forceinline__ void store4(double* p, const double (&v)[4]) {   // 32-byte aligned
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]),
+                 "d"(v[3])
+                 : "memory");
+}
+__device__ __forceinline__ void load4(const double* p, double (&v)[4]) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p)
+                 : "memory");
+}
+
+template <bool TF32, bool PAIR>
 __global__ void __launch_bounds__(THREADS, 1)
 k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__ err) {
     using F = Fmt<TF32>;
@@ -110,59 +140,93 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = (int64_t)g.mtiles * g.ntiles;
     volatile int32_t* verr = err;
+    constexpr int CTAS = PAIR ? 2 : 1;
+    const int rank = PAIR ? (int)cluster_rank() : 0;
+    const int64_t tile0 = blockIdx.x / CTAS, tstep = gridDim.x / CTAS;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < NSTAGE; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], EPI_WARPS); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], CTAS * EPI_WARPS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(tmem_slot)),
-                     "r"(TMEM_COLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(tmem_slot)),
+                         "r"(TMEM_COLS));
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(tmem_slot)),
+                         "r"(TMEM_COLS));
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        }
     }
     fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();   // both CTAs' barriers are there
     fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- TMA producer ----------------
-            const uint32_t bytes = 2u * A_TILE + 2u * (uint32_t)g.tn * ROW_BYTES;
+            const int bn = g.tn / CTAS;   // rows of B that this CTA holds
+            const uint32_t bytes = CTAS * (2u * A_TILE + 2u * (uint32_t)bn * ROW_BYTES);
             int stage = 0;
             uint32_t phase = 0;
             int32_t last_parity[NSTAGE];
             for (int i = 0; i < NSTAGE; ++i) last_parity[i] = -1;
             bool ok = true;
-            for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-                const int mt = (int)(tile % g.mtiles), nt = (int)(tile / g.mtiles);
+            for (int64_t tile = tile0; ok && tile < ntiles; tile += tstep) {
+                const int mt = tile_m(g, tile), nt = tile_n_of(g, tile);
                 for (int kb = 0; kb < g.kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, verr)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&full[stage], bytes);
-                    last_parity[stage] = (int32_t)phase;
+                    if (rank == 0) {
+                        mbar_arrive_expect_tx(&full[stage], bytes);
+                        last_parity[stage] = (int32_t)phase;
+                    }
                     const uint32_t st = smem_u32(stages + stage * STAGE_BYTES);
-                    const int k0 = kb * F::KE;
-                    tma_load_3d(st, &maps.a_hi, &full[stage], k0, mt * TM, 0);
-                    tma_load_3d(st + A_TILE, &maps.a_lo, &full[stage], k0, mt * TM, 0);
-                    tma_load_3d(st + 2 * A_TILE, &maps.b_hi, &full[stage], k0, nt * g.tn, 0);
-                    tma_load_3d(st + 2 * A_TILE + B_TILE, &maps.b_lo, &full[stage], k0, nt * g.tn, 0);
+                    const int k0 = kb * F::KE, ra = (mt * CTAS + rank) * TM, rb = nt * g.tn + rank * bn;
+                    if constexpr (PAIR) {
+                        const uint32_t bar = leader_bar(&full[stage]);
+                        tma_load_3d_pair(st, &maps.a_hi, bar, k0, ra, 0);
+                        tma_load_3d_pair(st + A_TILE, &maps.a_lo, bar, k0, ra, 0);
+                        tma_load_3d_pair(st + 2 * A_TILE, &maps.b_hi, bar, k0, rb, 0);
+                        tma_load_3d_pair(st + 2 * A_TILE + B_TILE, &maps.b_lo, bar, k0, rb, 0);
+                    } else {
+                        tma_load_3d(st, &maps.a_hi, &full[stage], k0, ra, 0);
+                        tma_load_3d(st + A_TILE, &maps.a_lo, &full[stage], k0, ra, 0);
+                        tma_load_3d(st + 2 * A_TILE, &maps.b_hi, &full[stage], k0, rb, 0);
+                        tma_load_3d(st + 2 * A_TILE + B_TILE, &maps.b_lo, &full[stage], k0, rb, 0);
+                    }
                     if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
                 }
             }
-            // drain: the copies of every issued stage land before the CTA exits
+            // drain: the copies of every issued stage (a pair's are counted by the leader)
+            // land before the CTA exits
             for (int i = 0; i < NSTAGE; ++i)
                 if (last_parity[i] >= 0) mbar_wait(&full[i], (uint32_t)last_parity[i], verr, false);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (lane == 0 && rank == 0) {
             // ---------------- MMA issuer ----------------
-            const uint32_t ID = F::ID | ((uint32_t)(g.tn >> 3) << 17);
+            const uint32_t ID = (F::ID + ((uint32_t)((CTAS - 1) * (TM >> 4)) << 24)) |
+                                ((uint32_t)(g.tn >> 3) << 17);
+            auto mma = [&](uint32_t d, uint32_t a, uint32_t b, uint32_t acc_on) {
+                if constexpr (TF32 && PAIR) mma_tf32_pair(d, sdesc(a), sdesc(b), ID, acc_on);
+                else if constexpr (TF32) mma_tf32(d, sdesc(a), sdesc(b), ID, acc_on);
+                else if constexpr (PAIR) mma_f16_pair(d, sdesc(a), sdesc(b), ID, acc_on);
+                else mma_f16(d, sdesc(a), sdesc(b), ID, acc_on);
+            };
+            auto commit = [&](uint64_t* bar) {
+                if constexpr (PAIR) mma_commit_pair(bar);
+                else mma_commit(bar);
+            };
             int stage = 0, acc = 0;
             uint32_t phase = 0, aphase = 0;
             bool ok = true;
-            for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+            for (int64_t tile = tile0; ok && tile < ntiles; tile += tstep) {
                 if (!mbar_wait(&tempty[acc], aphase ^ 1u, verr)) break;
                 fence_after();
                 const uint32_t dh = tmem + (uint32_t)acc * 256u, dx = dh + 128u;
@@ -176,57 +240,69 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
                     for (int kk = 0; kk < 2; ++kk) {   // 32 bytes of k per MMA
                         const uint32_t off = kk * 32;
                         const uint32_t first = (kb | kk) ? 1u : 0u;
-                        if constexpr (TF32) {
-                            mma_tf32(dh, sdesc(ah + off), sdesc(bh + off), ID, first);
-                            mma_tf32(dx, sdesc(ah + off), sdesc(bl + off), ID, first);
-                            mma_tf32(dx, sdesc(al + off), sdesc(bh + off), ID, 1u);
-                        } else {
-                            mma_f16(dh, sdesc(ah + off), sdesc(bh + off), ID, first);
-                            mma_f16(dx, sdesc(ah + off), sdesc(bl + off), ID, first);
-                            mma_f16(dx, sdesc(al + off), sdesc(bh + off), ID, 1u);
-                        }
+                        mma(dh, ah + off, bh + off, first);
+                        mma(dx, (g.lo_first ? al : ah) + off, (g.lo_first ? bh : bl) + off, first);
+                        mma(dx, (g.lo_first ? ah : al) + off, (g.lo_first ? bl : bh) + off, 1u);
                     }
-                    mma_commit(&empty[stage]);
+                    commit(&empty[stage]);
                     if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                mma_commit(&tfull[acc]);
+                commit(&tfull[acc]);
                 if (++acc == 2) { acc = 0; aphase ^= 1u; }
             }
         }
     } else {
-        // ---------------- epilogue (4 warps, one output row per thread) ----------------
+        // ---------------- epilogue (8 warps, half an output row per thread) ----------------
         const int quad = warp & 3;   // TMEM lanes this warp may read
+        const int half = (warp - 2) >> 2;   // every other 16 columns
         const int row = quad * 32 + lane;
         int acc = 0;
         uint32_t aphase = 0;
         E* ohi = (E*)g.out_hi;
         E* olo = (E*)g.out_lo;
-        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        for (int64_t tile = tile0; tile < ntiles; tile += tstep) {
             const bool bad = !mbar_wait(&tfull[acc], aphase, verr) || *verr;
             if (epi_any(bad)) break;
             fence_after();
-            const int mt = (int)(tile % g.mtiles), nt = (int)(tile / g.mtiles);
-            const int64_t m = (int64_t)mt * TM + row;
+            const int mt = tile_m(g, tile), nt = tile_n_of(g, tile);
+            const int64_t m = (int64_t)(mt * CTAS + rank) * TM + row;
             const bool mok = m < g.m;
             const int64_t ob = mok ? (m / g.kdiv) * g.rs_hi + (m % g.kdiv) * g.rs_lo : 0;
             const int c_base = nt * g.tn;
             const int ncols = min(g.tn, g.n - c_base);
             const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * 256u;
-            if (nt * g.tn < g.n && (int64_t)mt * TM + quad * 32 < g.m) {
+            // columns contiguous in memory: whole sectors of a thread's row
+            const bool vec = g.out && g.cs == 1 && ((uintptr_t)(g.out + ob + c_base) & 31) == 0;
+            if (nt * g.tn < g.n && (int64_t)(mt * CTAS + rank) * TM + quad * 32 < g.m) {
 #pragma unroll 1
-                for (int c0 = 0; c0 < ncols; c0 += 16) {
+                for (int c0 = 16 * half; c0 < ncols; c0 += 32) {
                     float xh[16], xx[16];
                     tmem_ld16(ta + c0, xh);
                     tmem_ld16(ta + 128u + c0, xx);
                     tmem_wait_ld();
-                    if (mok) {
+                    if (mok && vec && c0 + 16 <= ncols) {
+#pragma unroll
+                        for (int q = 0; q < 16; q += 4) {
+                            double* p = g.out + ob + c_base + c0 + q;
+                            double v[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) v[j] = double_of(xh[q + j]) + double_of(xx[q + j]);
+                            if (g.accumulate) {
+                                double w[4];
+                                load4(p, w);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) v[j] = w[j] + v[j];
+                            }
+                            store4(p, v);
+                        }
+                    } else if (mok) {
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             if (c0 + j < ncols) {
                                 const int64_t e = ob + (int64_t)(c_base + c0 + j) * g.cs;
                                 if (g.out) {
-                                    const double v = (double)xh[j] + (double)xx[j];
+                                    const double v = double_of(xh[j]) + double_of(xx[j]);
                                     g.out[e] = g.accumulate ? g.out[e] + v : v;
                                 } else {
                                     // hi.hi + cross as an exact FP32 pair (two-sum)
@@ -242,17 +318,25 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
             }
             fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[acc]);
+            if (lane == 0) {
+                if constexpr (PAIR) mbar_arrive_cluster(leader_bar(&tempty[acc]));
+                else mbar_arrive(&tempty[acc]);
+            }
             if (++acc == 2) { acc = 0; aphase ^= 1u; }
         }
     }
 
     fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();   // neither CTA's memory is in use any more
     fence_after();
     if (warp == 1) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(TMEM_COLS));
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                         "r"(TMEM_COLS));
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                         "r"(TMEM_COLS));
     }
 }
 
@@ -368,25 +452,30 @@ bool make_operand_map(CUtensorMap* m, bool tf32, const void* base, uint64_t kdim
     return r == CUDA_SUCCESS;
 }
 
-// N tile for n columns: the fewest tiles of at most 128, each a multiple of 16.
-int32_t tile_n(int32_t n) {
+// N tile for n columns: the fewest tiles of at most 128, each a multiple of `unit`.
+int32_t tile_n(int32_t n, int32_t unit) {
     const int32_t t = (n + 127) / 128;
-    return std::min(128, ((n + t - 1) / t + 15) / 16 * 16);
+    return std::min(128, ((n + t - 1) / t + unit - 1) / unit * unit);
 }
 
 template <bool TF32>
 int run_gemm(const void* a_hi, const void* a_lo, int64_t a_rows, const void* b_hi,
              const void* b_lo, int64_t b_rows, int32_t kdim, int32_t ld, int64_t kdiv,
              int64_t rs_hi, int64_t rs_lo, int64_t cs, double* out, void* out_hi, void* out_lo,
-             int32_t* err, cudaStream_t stream, bool accumulate = false) {
+             int32_t* err, cudaStream_t stream, bool accumulate = false, bool lo_first = false) {
     if (a_rows <= 0 || b_rows <= 0 || kdim <= 0) return CDS_OK;
     if (a_rows > INT32_MAX - TM) return CDS_ERR_ARG;
     Args g;
     g.m = (int32_t)a_rows;
     g.n = (int32_t)b_rows;
-    g.tn = tile_n(g.n);
+    // pairs of CTAs once every pair has a tile
+    const int sms = device_sms();
+    const int32_t tn2 = tile_n(g.n, 32);
+    const bool pair = (int64_t)((g.m + 2 * TM - 1) / (2 * TM)) * ((g.n + tn2 - 1) / tn2) >= sms / 2;
+    const int ctas = pair ? 2 : 1;
+    g.tn = pair ? tn2 : tile_n(g.n, 16);
     g.kblocks = (kdim + Fmt<TF32>::KE - 1) / Fmt<TF32>::KE;
-    g.mtiles = (g.m + TM - 1) / TM;
+    g.mtiles = (g.m + ctas * TM - 1) / (ctas * TM);
     g.ntiles = (g.n + g.tn - 1) / g.tn;
     g.kdiv = kdiv;
     g.rs_hi = rs_hi;
@@ -396,18 +485,31 @@ int run_gemm(const void* a_hi, const void* a_lo, int64_t a_rows, const void* b_h
     g.out_hi = out_hi;
     g.out_lo = out_lo;
     g.accumulate = accumulate ? 1 : 0;
+    g.lo_first = lo_first ? 1 : 0;
     Maps maps;
     if (!make_operand_map(&maps.a_hi, TF32, a_hi, kdim, a_rows, ld, TM) ||
         !make_operand_map(&maps.a_lo, TF32, a_lo, kdim, a_rows, ld, TM) ||
-        !make_operand_map(&maps.b_hi, TF32, b_hi, kdim, b_rows, ld, g.tn) ||
-        !make_operand_map(&maps.b_lo, TF32, b_lo, kdim, b_rows, ld, g.tn))
+        !make_operand_map(&maps.b_hi, TF32, b_hi, kdim, b_rows, ld, g.tn / ctas) ||
+        !make_operand_map(&maps.b_lo, TF32, b_lo, kdim, b_rows, ld, g.tn / ctas))
         return CDS_ERR_CUDA;
-    // per launch: the attribute belongs to the current device
-    CDS_CUDA_TRY(cudaFuncSetAttribute(k_tr_gemm<TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)SMEM_BYTES));
     const int64_t tiles = (int64_t)g.mtiles * g.ntiles;
-    const int grid = (int)std::min<int64_t>(tiles, device_sms());
-    k_tr_gemm<TF32><<<grid, THREADS, SMEM_BYTES, stream>>>(maps, g, err);
+    auto kern = pair ? k_tr_gemm<TF32, true> : k_tr_gemm<TF32, false>;
+    // per launch: the attribute belongs to the current device
+    CDS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)SMEM_BYTES));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(tiles * ctas, sms / ctas * ctas));
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const Maps&)maps, (const Args&)g, err));
     CDS_LAUNCH_CHECK();
     return CDS_OK;
 }
@@ -486,15 +588,15 @@ int batch(int32_t N, int32_t nmo, int32_t nocc, int32_t np, const double* L, con
 int tr_split_gemm(int32_t precision, const void* a_hi, const void* a_lo, int64_t a_rows,
                   const void* b_hi, const void* b_lo, int64_t b_rows, int32_t kdim, int32_t ld,
                   int64_t kdiv, int64_t rs_hi, int64_t rs_lo, int64_t cs, double* out,
-                  bool accumulate, int32_t* err, cudaStream_t stream) {
+                  bool accumulate, int32_t* err, cudaStream_t stream, bool lo_first) {
     if (!tc::device_ok()) return CDS_ERR_UNSUPPORTED;
     if (!out || kdiv <= 0 || ld < kdim) return CDS_ERR_ARG;
     if (precision == CDS_PREC_TF32X3)
         return trc::run_gemm<true>(a_hi, a_lo, a_rows, b_hi, b_lo, b_rows, kdim, ld, kdiv, rs_hi,
-                                   rs_lo, cs, out, nullptr, nullptr, err, stream, accumulate);
+                                   rs_lo, cs, out, nullptr, nullptr, err, stream, accumulate, lo_first);
     if (precision == CDS_PREC_BF16X3)
         return trc::run_gemm<false>(a_hi, a_lo, a_rows, b_hi, b_lo, b_rows, kdim, ld, kdiv, rs_hi,
-                                    rs_lo, cs, out, nullptr, nullptr, err, stream, accumulate);
+                                    rs_lo, cs, out, nullptr, nullptr, err, stream, accumulate, lo_first);
     return CDS_ERR_UNSUPPORTED;
 }
 

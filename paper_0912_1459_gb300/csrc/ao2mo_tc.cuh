@@ -29,11 +29,12 @@ int tr_tc_status(int32_t nbf, int32_t nmo, int32_t nocc, int32_t np, int32_t kb_
 // elements, 16-byte aligned rows), a_rows x kdim and b_rows x kdim; FP64
 // output element (m, c) at out[(m / kdiv) rs_hi + (m % kdiv) rs_lo + c cs],
 // written or (accumulate) added.  Asynchronous; the kernel's error word is
-// err (device int32, cleared by the caller).
+// err (device int32, cleared by the caller).  lo_first: the cross products as lo.hi +
+// hi.lo, i.e. the result of the call with A and B exchanged, bit for bit.
 int tr_split_gemm(int32_t precision, const void* a_hi, const void* a_lo, int64_t a_rows,
                   const void* b_hi, const void* b_lo, int64_t b_rows, int32_t kdim, int32_t ld,
                   int64_t kdiv, int64_t rs_hi, int64_t rs_lo, int64_t cs, double* out,
-                  bool accumulate, int32_t* err, cudaStream_t stream);
+                  bool accumulate, int32_t* err, cudaStream_t stream, bool lo_first = false);
 
 // Exact-slice (Ozaki) form, CDS_PREC_OZAKI: nbf <= 1040.
 size_t tr_oz_workspace_bytes(int32_t nbf, int32_t nmo, int32_t nocc, int32_t np, int32_t kb_max);

@@ -106,6 +106,19 @@ __device__ __forceinline__ double eri_pair(double p, double px, double py, doubl
     return eri_is_far(x, s) ? eri_far(kp * kq, x) : eri_near(kp * kq, x, s);
 }
 
+// (double)x in integer operations (a branch-free conversion): the conversions between
+// float and double run on the FP64 units, at one a clock and SM or less.
+__device__ __forceinline__ double double_of(float x) {
+    const bool tiny = fabsf(x) < 0x1p-100f;                        // subnormals among them
+    const uint32_t b = __float_as_uint(tiny ? x * 0x1p64f : x), m = b & 0x7fffffffu;
+    uint32_t hi = (m >> 3) + (tiny ? (896u - 64u) << 20 : 896u << 20);
+    if (m == 0u) hi = 0u;
+    if (m >= 0x7f800000u) hi += 896u << 20;                        // infinite, NaN
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+// The double of a float pair.
+__device__ __forceinline__ double double_of(float2 v) { return double_of(v.x) + double_of(v.y); }
+
 // Decode a packed pair index I = nu(nu+1)/2 + mu into (mu, nu).
 __device__ __forceinline__ void unpack_pair(int64_t I, int32_t& mu, int32_t& nu) {
     double r = sqrt(8.0 * (double)I + 1.0);
