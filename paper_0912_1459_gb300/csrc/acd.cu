@@ -115,7 +115,7 @@ template <bool DF>
 __device__ __forceinline__ double x_at(const double* B, const float2* Xf, int64_t e) {
     if (DF) {
         const float2 v = Xf[e];
-        return (double)v.x + (double)v.y;
+        return double_of(v);
     }
     return B[e];
 }

@@ -135,7 +135,7 @@ __device__ __forceinline__ void df_fma(float2& acc, float2 a, float2 b) {
     acc.y += err + pe;
 }
 
-__device__ __forceinline__ void store_out(double* p, float2 v) { p[0] = (double)v.x + (double)v.y; }
+__device__ __forceinline__ void store_out(double* p, float2 v) { p[0] = double_of(v); }
 __device__ __forceinline__ void store_out(float2* p, float2 v) {
     const float h = v.x + v.y;
     p[0] = make_float2(h, v.y - (h - v.x));

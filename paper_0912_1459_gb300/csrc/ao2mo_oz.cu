@@ -333,7 +333,7 @@ k_oz_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
                         if (8 * c < hw && col < g.n) {
                             const float st = sa * g.sb[col];   // power of two
                             const int64_t e = ob + (int64_t)col * g.cs;
-                            if (g.out) g.out[e] = (double)(v[c][j].x * st) + (double)(v[c][j].y * st);
+                            if (g.out) g.out[e] = double_of(make_float2(v[c][j].x * st, v[c][j].y * st));
                             else g.outf[e] = make_float2(v[c][j].x * st, v[c][j].y * st);
                         }
                     }

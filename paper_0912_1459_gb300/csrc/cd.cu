@@ -455,9 +455,19 @@ __global__ void k_cd_tc_scales(const double* __restrict__ D, int64_t n, float* _
 // The digit slices of x / sigma (sigma = 2^e > |x|), x a float pair:
 // q = trunc(x 2^(Q-e)) (|q| < 2^Q, Q = 56 bits), digit s = bits
 // [Q-7(s+1), Q-7s) of |q|, slice s = sign(x) digit 2^(-7(s+1)) (exact in BF16).
+// In integer operations: conversions to 64-bit integers run on the FP64 units.
+__device__ __forceinline__ long long tc_fixed(float x, int e) {   // trunc(x 2^(Q - e)), up to 2^62
+    const uint32_t b = __float_as_uint(x);
+    const int ex = (int)((b >> 23) & 255u);
+    const uint32_t m = (b & 0x7fffffu) | (ex ? 0x800000u : 0u);    // x = m 2^(max(ex, 1) - 150)
+    const int sh = max(ex, 1) - 150 + kSlicesTC * kBitsTC - e;
+    const unsigned long long q = sh >= 0 ? (unsigned long long)m << min(sh, 38)
+                                         : (unsigned long long)(sh > -32 ? m >> -sh : 0u);
+    return b >> 31 ? -(long long)q : (long long)q;
+}
 __device__ __forceinline__ void tc_slices(float2 x, int e, uint16_t (&out)[kSlicesTC]) {
     constexpr int QB = kSlicesTC * kBitsTC;
-    long long q = __float2ll_rz(ldexpf(x.x, QB - e)) + __float2ll_rz(ldexpf(x.y, QB - e));
+    long long q = tc_fixed(x.x, e) + tc_fixed(x.y, e);
     const long long qmax = (1LL << QB) - 1;
     q = q > qmax ? qmax : (q < -qmax ? -qmax : q);
     const bool neg = q < 0;
@@ -465,8 +475,8 @@ __device__ __forceinline__ void tc_slices(float2 x, int e, uint16_t (&out)[kSlic
 #pragma unroll
     for (int s = 0; s < kSlicesTC; ++s) {
         const int d = (int)((aq >> (QB - kBitsTC * (s + 1))) & ((1ull << kBitsTC) - 1));
-        out[s] = __bfloat16_as_ushort(__float2bfloat16_rn(ldexpf((float)(neg ? -d : d),
-                                                                 -kBitsTC * (s + 1))));
+        const float f = __int_as_float(0x4B400000 + (neg ? -d : d)) - 12582912.f;   // (float)d
+        out[s] = (uint16_t)(__float_as_uint(f * __int_as_float((127 - kBitsTC * (s + 1)) << 23)) >> 16);
     }
 }
 
@@ -647,13 +657,13 @@ __device__ __forceinline__ void cd_step_body(int64_t n, int32_t k, int32_t max_r
                 const float2 lf = df_mul(df_add(e, df_neg(acc)), rDPf);
                 *reinterpret_cast<float2*>(slot) = lf;
                 const float2 l2 = df_mul(lf, lf);
-                d = D[I] - ((double)l2.x + (double)l2.y);
+                d = D[I] - double_of(l2);
             } else {
                 double proj = 0.0;
                 if (k > 0) {
                     if constexpr (DF) {
                         const float2 f = *reinterpret_cast<const float2*>(slot);
-                        proj = (double)f.x + (double)f.y;
+                        proj = double_of(f);
                     } else {
                         proj = *slot;
                     }
@@ -1108,7 +1118,7 @@ k_screen_spread(const float2* __restrict__ Lc, int64_t nc, const int32_t* __rest
         const int32_t j = inv[I];
         const float2 v = j >= 0 ? Lc[r * nc + j] : make_float2(0.f, 0.f);
         if (PAIRS) reinterpret_cast<float2*>(L)[r * n + I] = v;
-        else L[r * n + I] = (double)v.x + (double)v.y;
+        else L[r * n + I] = double_of(v);
     }
 }
 
@@ -1127,7 +1137,7 @@ __global__ void k_pairs_to_fp64(double* __restrict__ L, int64_t count) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= count) return;
     const float2 v = reinterpret_cast<const float2*>(L)[i];
-    L[i] = (double)v.x + (double)v.y;
+    L[i] = double_of(v);
 }
 
 }  // namespace cds
@@ -2195,7 +2205,7 @@ __global__ void k_bcd_tc_scatter(const float2* __restrict__ Lc, int64_t nc,
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = i / nc, j = i - r * nc;
         const float2 v = Lc[i];
-        L[r * n + live[j]] = (double)v.x + (double)v.y;
+        L[r * n + live[j]] = double_of(v);
     }
 }
 

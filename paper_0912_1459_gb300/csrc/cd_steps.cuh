@@ -310,7 +310,7 @@ __device__ __forceinline__ void cd_steps_body(const CdStepsArgs& a, int cta, int
                         if (RES && extra < a.srows)
                             s_row[(int64_t)extra * np + sb * kStepChunk + q * kUpdThreads + tt] = lf[q];
                         const float2 l2 = df_mul(lf[q], lf[q]);
-                        double d = (RES ? dreg[q] : a.D[I]) - ((double)l2.x + (double)l2.y);
+                        double d = (RES ? dreg[q] : a.D[I]) - double_of(l2);
                         if (I == P) d = 0.0;
                         if (RES) dreg[q] = d;
                         else a.D[I] = d;
