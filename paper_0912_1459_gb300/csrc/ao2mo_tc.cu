@@ -20,9 +20,7 @@
 //
 // One kernel serves the three GEMMs: D[m][n] = sum_k A[m][k] B[n][k], both
 // operands K-major (k contiguous), a persistent grid walking the tiles of 128 x tn
-// (tn <= 128, a multiple of 16), or, once there are enough tiles for every pair of
-// SMs, of 256 x tn (a multiple of 32) by two CTAs each, which halves what B takes of
-// the shared memory's and the L2's bandwidth.  Warp 0 = TMA producer, warp 1 =
+// (tn <= 128, a multiple of 16).  Warp 0 = TMA producer, warp 1 =
 // TMEM allocator + MMA issuer, warps 2..9 = epilogue (half an output row per
 // thread).  Shared memory holds NSTAGE stages of {A_hi, A_lo, B_hi, B_lo}
 // (rows of 64 bytes, 64-byte swizzle); TMEM holds two accumulator pairs so
@@ -31,9 +29,11 @@
 //
 // What bounds it: with few k the epilogue, until its conversions to FP64 (one a clock
 // and SM) became integer operations, 660 x 118,800 outputs of K = 896 0.81 -> 0.46 ms;
-// with many k the operands' delivery, 5,280 x 896 of K = 118,800 2.6 ms (1.3 PFLOP/s).
-// Walking the side with fewer tiles first reads the larger operand from DRAM once:
-// 118,800 x 896 of K = 5,280 3.2 -> 2.6 ms.
+// with many k the shared memory's port, which the MMAs' operands and the TMA's writes
+// share: 640 clocks per k-block, 576 with the wide MMA below, for 384 of arithmetic
+// (5,280 x 896 of K = 118,800 2.55 ms, 1.3 PFLOP/s; tiles of 256 rows by pairs of CTAs,
+// with less of that traffic, were no faster).  Walking the side with fewer tiles first
+// reads the larger operand from DRAM once: 118,800 x 896 of K = 5,280 3.2 -> 2.45 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -122,7 +122,7 @@ __device__ __forceinline__ void load4(const double* p, double (&v)[4]) {
                  : "memory");
 }
 
-template <bool TF32, bool PAIR>
+template <bool TF32>
 __global__ void __launch_bounds__(THREADS, 1)
 k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__ err) {
     using F = Fmt<TF32>;
@@ -140,115 +140,97 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = (int64_t)g.mtiles * g.ntiles;
     volatile int32_t* verr = err;
-    constexpr int CTAS = PAIR ? 2 : 1;
-    const int rank = PAIR ? (int)cluster_rank() : 0;
-    const int64_t tile0 = blockIdx.x / CTAS, tstep = gridDim.x / CTAS;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < NSTAGE; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], CTAS * EPI_WARPS); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], EPI_WARPS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        if constexpr (PAIR) {
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                             smem_u32(tmem_slot)),
-                         "r"(TMEM_COLS));
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                             smem_u32(tmem_slot)),
-                         "r"(TMEM_COLS));
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-        }
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync();   // both CTAs' barriers are there
     fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- TMA producer ----------------
-            const int bn = g.tn / CTAS;   // rows of B that this CTA holds
-            const uint32_t bytes = CTAS * (2u * A_TILE + 2u * (uint32_t)bn * ROW_BYTES);
+            const uint32_t bytes = 2u * A_TILE + 2u * (uint32_t)g.tn * ROW_BYTES;
             int stage = 0;
             uint32_t phase = 0;
             int32_t last_parity[NSTAGE];
             for (int i = 0; i < NSTAGE; ++i) last_parity[i] = -1;
             bool ok = true;
-            for (int64_t tile = tile0; ok && tile < ntiles; tile += tstep) {
+            for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
                 const int mt = tile_m(g, tile), nt = tile_n_of(g, tile);
                 for (int kb = 0; kb < g.kblocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, verr)) { ok = false; break; }
-                    if (rank == 0) {
-                        mbar_arrive_expect_tx(&full[stage], bytes);
-                        last_parity[stage] = (int32_t)phase;
-                    }
+                    mbar_arrive_expect_tx(&full[stage], bytes);
+                    last_parity[stage] = (int32_t)phase;
                     const uint32_t st = smem_u32(stages + stage * STAGE_BYTES);
-                    const int k0 = kb * F::KE, ra = (mt * CTAS + rank) * TM, rb = nt * g.tn + rank * bn;
-                    if constexpr (PAIR) {
-                        const uint32_t bar = leader_bar(&full[stage]);
-                        tma_load_3d_pair(st, &maps.a_hi, bar, k0, ra, 0);
-                        tma_load_3d_pair(st + A_TILE, &maps.a_lo, bar, k0, ra, 0);
-                        tma_load_3d_pair(st + 2 * A_TILE, &maps.b_hi, bar, k0, rb, 0);
-                        tma_load_3d_pair(st + 2 * A_TILE + B_TILE, &maps.b_lo, bar, k0, rb, 0);
-                    } else {
-                        tma_load_3d(st, &maps.a_hi, &full[stage], k0, ra, 0);
-                        tma_load_3d(st + A_TILE, &maps.a_lo, &full[stage], k0, ra, 0);
-                        tma_load_3d(st + 2 * A_TILE, &maps.b_hi, &full[stage], k0, rb, 0);
-                        tma_load_3d(st + 2 * A_TILE + B_TILE, &maps.b_lo, &full[stage], k0, rb, 0);
-                    }
+                    const int k0 = kb * F::KE;
+                    tma_load_3d(st, &maps.a_hi, &full[stage], k0, mt * TM, 0);
+                    tma_load_3d(st + A_TILE, &maps.a_lo, &full[stage], k0, mt * TM, 0);
+                    tma_load_3d(st + 2 * A_TILE, &maps.b_hi, &full[stage], k0, nt * g.tn, 0);
+                    tma_load_3d(st + 2 * A_TILE + g.tn * ROW_BYTES, &maps.b_lo, &full[stage], k0,
+                                nt * g.tn, 0);
                     if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
                 }
             }
-            // drain: the copies of every issued stage (a pair's are counted by the leader)
-            // land before the CTA exits
+            // drain: the copies of every issued stage land before the CTA exits
             for (int i = 0; i < NSTAGE; ++i)
                 if (last_parity[i] >= 0) mbar_wait(&full[i], (uint32_t)last_parity[i], verr, false);
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (lane == 0) {
             // ---------------- MMA issuer ----------------
-            const uint32_t ID = (F::ID + ((uint32_t)((CTAS - 1) * (TM >> 4)) << 24)) |
-                                ((uint32_t)(g.tn >> 3) << 17);
-            auto mma = [&](uint32_t d, uint32_t a, uint32_t b, uint32_t acc_on) {
-                if constexpr (TF32 && PAIR) mma_tf32_pair(d, sdesc(a), sdesc(b), ID, acc_on);
-                else if constexpr (TF32) mma_tf32(d, sdesc(a), sdesc(b), ID, acc_on);
-                else if constexpr (PAIR) mma_f16_pair(d, sdesc(a), sdesc(b), ID, acc_on);
-                else mma_f16(d, sdesc(a), sdesc(b), ID, acc_on);
-            };
-            auto commit = [&](uint64_t* bar) {
-                if constexpr (PAIR) mma_commit_pair(bar);
-                else mma_commit(bar);
+            // hi.hi and one cross product by one MMA of 2 tn columns: B's hi and lo rows
+            // follow each other, as the accumulators do, and A is read once for both
+            const uint32_t ID = F::ID | ((uint32_t)(g.tn >> 3) << 17);
+            const uint32_t IDw = F::ID | ((uint32_t)(g.tn >> 2) << 17);
+            auto mma = [&](uint32_t d, uint32_t a, uint32_t b, uint32_t id, uint32_t acc_on) {
+                if constexpr (TF32) mma_tf32(d, sdesc(a), sdesc(b), id, acc_on);
+                else mma_f16(d, sdesc(a), sdesc(b), id, acc_on);
             };
             int stage = 0, acc = 0;
             uint32_t phase = 0, aphase = 0;
             bool ok = true;
-            for (int64_t tile = tile0; ok && tile < ntiles; tile += tstep) {
+            for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
                 if (!mbar_wait(&tempty[acc], aphase ^ 1u, verr)) break;
                 fence_after();
-                const uint32_t dh = tmem + (uint32_t)acc * 256u, dx = dh + 128u;
+                const uint32_t dh = tmem + (uint32_t)acc * 256u, dx = dh + (uint32_t)g.tn;
                 for (int kb = 0; kb < g.kblocks; ++kb) {
                     if (!mbar_wait(&full[stage], phase, verr)) { ok = false; break; }
                     fence_after();
                     const uint32_t base = smem_u32(stages + stage * STAGE_BYTES);
                     const uint32_t ah = base, al = base + A_TILE;
-                    const uint32_t bh = base + 2 * A_TILE, bl = bh + B_TILE;
+                    const uint32_t bh = base + 2 * A_TILE, bl = bh + (uint32_t)(g.tn * ROW_BYTES);
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk) {   // 32 bytes of k per MMA
                         const uint32_t off = kk * 32;
                         const uint32_t first = (kb | kk) ? 1u : 0u;
-                        mma(dh, ah + off, bh + off, first);
-                        mma(dx, (g.lo_first ? al : ah) + off, (g.lo_first ? bh : bl) + off, first);
-                        mma(dx, (g.lo_first ? ah : al) + off, (g.lo_first ? bl : bh) + off, 1u);
+                        if (g.lo_first && first == 0u) {   // (the wide MMA starts both sums)
+                            mma(dh, ah + off, bh + off, ID, 0u);
+                            mma(dx, al + off, bh + off, ID, 0u);
+                            mma(dx, ah + off, bl + off, ID, 1u);
+                        } else if (g.lo_first) {
+                            mma(dx, al + off, bh + off, ID, 1u);
+                            mma(dh, ah + off, bh + off, IDw, 1u);
+                        } else {
+                            mma(dh, ah + off, bh + off, IDw, first);
+                            mma(dx, al + off, bh + off, ID, 1u);
+                        }
                     }
-                    commit(&empty[stage]);
+                    mma_commit(&empty[stage]);
                     if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
-                commit(&tfull[acc]);
+                mma_commit(&tfull[acc]);
                 if (++acc == 2) { acc = 0; aphase ^= 1u; }
             }
         }
@@ -261,12 +243,12 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
         uint32_t aphase = 0;
         E* ohi = (E*)g.out_hi;
         E* olo = (E*)g.out_lo;
-        for (int64_t tile = tile0; tile < ntiles; tile += tstep) {
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             const bool bad = !mbar_wait(&tfull[acc], aphase, verr) || *verr;
             if (epi_any(bad)) break;
             fence_after();
             const int mt = tile_m(g, tile), nt = tile_n_of(g, tile);
-            const int64_t m = (int64_t)(mt * CTAS + rank) * TM + row;
+            const int64_t m = (int64_t)mt * TM + row;
             const bool mok = m < g.m;
             const int64_t ob = mok ? (m / g.kdiv) * g.rs_hi + (m % g.kdiv) * g.rs_lo : 0;
             const int c_base = nt * g.tn;
@@ -274,12 +256,12 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
             const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * 256u;
             // columns contiguous in memory: whole sectors of a thread's row
             const bool vec = g.out && g.cs == 1 && ((uintptr_t)(g.out + ob + c_base) & 31) == 0;
-            if (nt * g.tn < g.n && (int64_t)(mt * CTAS + rank) * TM + quad * 32 < g.m) {
+            if (nt * g.tn < g.n && (int64_t)mt * TM + quad * 32 < g.m) {
 #pragma unroll 1
                 for (int c0 = 16 * half; c0 < ncols; c0 += 32) {
                     float xh[16], xx[16];
                     tmem_ld16(ta + c0, xh);
-                    tmem_ld16(ta + 128u + c0, xx);
+                    tmem_ld16(ta + (uint32_t)g.tn + c0, xx);
                     tmem_wait_ld();
                     if (mok && vec && c0 + 16 <= ncols) {
 #pragma unroll
@@ -318,25 +300,17 @@ k_tr_gemm(const __grid_constant__ Maps maps, const Args g, int32_t* __restrict__
             }
             fence_before();
             __syncwarp();
-            if (lane == 0) {
-                if constexpr (PAIR) mbar_arrive_cluster(leader_bar(&tempty[acc]));
-                else mbar_arrive(&tempty[acc]);
-            }
+            if (lane == 0) mbar_arrive(&tempty[acc]);
             if (++acc == 2) { acc = 0; aphase ^= 1u; }
         }
     }
 
     fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync();   // neither CTA's memory is in use any more
     fence_after();
     if (warp == 1) {
-        if constexpr (PAIR)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                         "r"(TMEM_COLS));
-        else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                         "r"(TMEM_COLS));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(TMEM_COLS));
     }
 }
 
@@ -452,10 +426,10 @@ bool make_operand_map(CUtensorMap* m, bool tf32, const void* base, uint64_t kdim
     return r == CUDA_SUCCESS;
 }
 
-// N tile for n columns: the fewest tiles of at most 128, each a multiple of `unit`.
-int32_t tile_n(int32_t n, int32_t unit) {
+// N tile for n columns: the fewest tiles of at most 128, each a multiple of 16.
+int32_t tile_n(int32_t n) {
     const int32_t t = (n + 127) / 128;
-    return std::min(128, ((n + t - 1) / t + unit - 1) / unit * unit);
+    return std::min(128, ((n + t - 1) / t + 15) / 16 * 16);
 }
 
 template <bool TF32>
@@ -468,14 +442,9 @@ int run_gemm(const void* a_hi, const void* a_lo, int64_t a_rows, const void* b_h
     Args g;
     g.m = (int32_t)a_rows;
     g.n = (int32_t)b_rows;
-    // pairs of CTAs once every pair has a tile
-    const int sms = device_sms();
-    const int32_t tn2 = tile_n(g.n, 32);
-    const bool pair = (int64_t)((g.m + 2 * TM - 1) / (2 * TM)) * ((g.n + tn2 - 1) / tn2) >= sms / 2;
-    const int ctas = pair ? 2 : 1;
-    g.tn = pair ? tn2 : tile_n(g.n, 16);
+    g.tn = tile_n(g.n);
     g.kblocks = (kdim + Fmt<TF32>::KE - 1) / Fmt<TF32>::KE;
-    g.mtiles = (g.m + ctas * TM - 1) / (ctas * TM);
+    g.mtiles = (g.m + TM - 1) / TM;
     g.ntiles = (g.n + g.tn - 1) / g.tn;
     g.kdiv = kdiv;
     g.rs_hi = rs_hi;
@@ -489,27 +458,15 @@ int run_gemm(const void* a_hi, const void* a_lo, int64_t a_rows, const void* b_h
     Maps maps;
     if (!make_operand_map(&maps.a_hi, TF32, a_hi, kdim, a_rows, ld, TM) ||
         !make_operand_map(&maps.a_lo, TF32, a_lo, kdim, a_rows, ld, TM) ||
-        !make_operand_map(&maps.b_hi, TF32, b_hi, kdim, b_rows, ld, g.tn / ctas) ||
-        !make_operand_map(&maps.b_lo, TF32, b_lo, kdim, b_rows, ld, g.tn / ctas))
+        !make_operand_map(&maps.b_hi, TF32, b_hi, kdim, b_rows, ld, g.tn) ||
+        !make_operand_map(&maps.b_lo, TF32, b_lo, kdim, b_rows, ld, g.tn))
         return CDS_ERR_CUDA;
-    const int64_t tiles = (int64_t)g.mtiles * g.ntiles;
-    auto kern = pair ? k_tr_gemm<TF32, true> : k_tr_gemm<TF32, false>;
     // per launch: the attribute belongs to the current device
-    CDS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    CDS_CUDA_TRY(cudaFuncSetAttribute(k_tr_gemm<TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)SMEM_BYTES));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>(tiles * ctas, sms / ctas * ctas));
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)ctas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    CDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const Maps&)maps, (const Args&)g, err));
+    const int64_t tiles = (int64_t)g.mtiles * g.ntiles;
+    const int grid = (int)std::min<int64_t>(tiles, device_sms());
+    k_tr_gemm<TF32><<<grid, THREADS, SMEM_BYTES, stream>>>(maps, g, err);
     CDS_LAUNCH_CHECK();
     return CDS_OK;
 }

@@ -1,6 +1,5 @@
-"""The split products' GEMM where its tiles change: one CTA per tile of 128 rows against
-two per tile of 256 (enough tiles for every pair of SMs), a last tile of which one CTA's
-half is empty, widths that are rounded up to 16 or 32 columns, several tiles of columns.
+"""The split products' GEMM where its tiles change: one tile and many, last tiles that are
+nearly empty, widths that are rounded up to 16 columns, several tiles of columns.
 
 Each operand is hi + lo to 2^-17 (BF16X3) or 2^-22 (TF32X3) of itself, the lo.lo product
 is dropped and sums are FP32: with u twice that a product is off by at most 4 u |a||b|
@@ -23,10 +22,10 @@ DEV = torch.device("cuda:0")
 @pytest.mark.parametrize("precision,u", [("bf16x3", 2.0 ** -16), ("tf32x3", 2.0 ** -21)])
 @pytest.mark.parametrize("N,M,o,np_", [
     (5, 3, 2, 1),        # one tile, 16 columns
-    (60, 40, 17, 3),     # 2,400 rows: single CTAs
-    (96, 203, 17, 16),   # 19,488 rows: 77 pairs of tiles, one CTA of the last half empty
-    (96, 204, 30, 3),    # 33 columns: two tiles of 32
-    (130, 160, 64, 66),  # 130 columns
+    (60, 40, 17, 3),     # 2,400 rows: fewer tiles than SMs
+    (96, 203, 17, 16),   # 19,488 rows: 32 rows in the last tile; 33 columns
+    (96, 204, 30, 3),
+    (130, 160, 64, 66),  # 130 columns: two tiles of 80
     (200, 128, 60, 1),
 ])
 def test_against_fp64(precision, u, N, M, o, np_):
