@@ -41,8 +41,39 @@ inline int32_t ld8(int64_t n) { return (int32_t)((n + 7) / 8 * 8); }   // 16-byt
 template <bool TF32>
 using E = trc::SplitE<TF32>;
 
+// The BF16 split of x through its float pair, packed lo << 16 | hi, in integer
+// operations: f = x rounded to 24 bits, r = the remainder rounded to 24, hi =
+// bf16(f), lo = bf16((f - hi) + r).  The conversions it stands for run on the FP64
+// pipe, two a clock and SM.  False outside 2^-74 .. 2^126 (and for 0, inf, NaN).
+__device__ __forceinline__ bool split_bits(double x, uint32_t& packed) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ffull);
+    if ((unsigned)(ex - 949) > 200u) return false;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+    unsigned F = (unsigned)(m >> 29);
+    const unsigned low = (unsigned)m & 0x1fffffffu;
+    F += (low > 0x10000000u || (low == 0x10000000u && (F & 1u))) ? 1u : 0u;
+    int rem = (int)((unsigned)m - (F << 29));      // m - F 2^29, |rem| <= 2^28
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+    if (sign) rem = -rem;
+    const float f = __uint_as_float(sign | (((uint32_t)(ex - 896) << 23) + (F - 0x800000u)));
+    const float r = (float)rem * __int_as_float((ex - 948) << 23);
+    uint16_t h, l;
+    trc::split_bf16(f, r, h, l);
+    packed = (uint32_t)h | ((uint32_t)l << 16);
+    return true;
+}
+
 template <bool TF32>
 __device__ __forceinline__ void split_d(double x, E<TF32>* hi, E<TF32>* lo, int64_t e) {
+    if constexpr (!TF32) {
+        uint32_t pk;
+        if (split_bits(x, pk)) {
+            hi[e] = (E<TF32>)(uint16_t)pk;
+            lo[e] = (E<TF32>)(uint16_t)(pk >> 16);
+            return;
+        }
+    }
     float f, r;
     trc::pair_of_double(x, f, r);
     trc::split_store<TF32>(f, r, hi, lo, e);
@@ -97,29 +128,6 @@ struct GxArgs {
     void *ga_hi, *ga_lo, *gb_hi, *gb_lo;
 };
 
-// The BF16 split of x as split_d makes it, packed lo << 16 | hi, in integer
-// operations: f = x rounded to 24 bits, r = the remainder rounded to 24, hi =
-// bf16(f), lo = bf16((f - hi) + r).  The conversions it stands for run on the FP64
-// pipe, two a clock and SM.  False outside 2^-74 .. 2^126 (and for 0, inf, NaN).
-__device__ __forceinline__ bool split_bits(double x, uint32_t& packed) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7ffull);
-    if ((unsigned)(ex - 949) > 200u) return false;
-    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
-    unsigned F = (unsigned)(m >> 29);
-    const unsigned low = (unsigned)m & 0x1fffffffu;
-    F += (low > 0x10000000u || (low == 0x10000000u && (F & 1u))) ? 1u : 0u;
-    int rem = (int)((unsigned)m - (F << 29));      // m - F 2^29, |rem| <= 2^28
-    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-    if (sign) rem = -rem;
-    const float f = __uint_as_float(sign | (((uint32_t)(ex - 896) << 23) + (F - 0x800000u)));
-    const float r = (float)rem * __int_as_float((ex - 948) << 23);
-    uint16_t h, l;
-    trc::split_bf16(f, r, h, l);
-    packed = (uint32_t)h | ((uint32_t)l << 16);
-    return true;
-}
-
 // 1 / d to within 1 ulp: the PTX reciprocal seed and one cubic Newton step; zero,
 // subnormal, infinite and NaN d take the plain division.
 __device__ __forceinline__ double recip(double d) {
@@ -149,7 +157,7 @@ __device__ __forceinline__ double warp_sums4(const double (&v)[4]) {
 // operations per element here (7 for D, its reciprocal, G and r, 2.4 for the sums
 // over x, c2 and c1, which meet across the warp once per kC1 tiles), 60 with
 // divisions, a warp sum per row and the splits' conversions on that pipe too
-// (60.6 ms of an 80.2 ms gradient of 8 orbitals of 840 functions; 18.4 of 32.7 now).
+// (60.6 ms of an 80.2 ms gradient of 8 orbitals of 840 functions; 18.3 of 31.1 now).
 constexpr int kC1 = 4;
 template <bool TF32>
 __global__ void __launch_bounds__(256)
