@@ -355,7 +355,8 @@ int cds_ri_factors(int32_t nbf, const double* xyz, const double* alpha, const in
  * Blocking, like cds_cd_decompose.  The two library streams belong to the
  * device, so calls from several host threads share them (their work
  * interleaves in stream order).  On the library stream the tensor-core
- * decomposition replays its 32-step chunks as a CUDA graph (CDS_TUNE_CD_GRAPH);
+ * decomposition replays the passes between two host checks as a CUDA graph
+ * (CDS_TUNE_CD_GRAPH);
  * CDS_TUNE_PIPE_SPLIT divides the SMs between the two streams.
  * ---------------------------------------------------------------------- */
 size_t cds_cd_decompose_to_mo_workspace_bytes(int32_t nbf, int32_t nmo, int32_t nocc,
@@ -595,8 +596,9 @@ size_t cds_batch_workspace_bytes(int32_t nmol, const cds_mol* mols, int32_t prec
 /* Blocking.  Per molecule as cds_cd_decompose (delta and scheme shared);
  * M_out: host [nmol].  precision: CDS_PREC_FP64, or CDS_PREC_F32X2 (float-pair
  * projections and vectors, FP64 integral column, residuals and pivot
- * decisions; L converted to FP64 at the end): one update and one
- * pivot-select launch per step for the whole batch.  CDS_PREC_OZAKI: the
+ * decisions; L converted to FP64 at the end): two launches per step for the
+ * whole batch (FP64 with its region of the workspace: one launch per group of
+ * molecules).  CDS_PREC_OZAKI: the
  * tensor-core form of cds_cd_decompose for every molecule (the same
  * screening, pivots and arithmetic, so the same results bit for bit), its
  * steps batched: three launches per step (slicing, projection GEMM, update)

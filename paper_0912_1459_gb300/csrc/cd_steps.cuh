@@ -30,8 +30,9 @@
 // Every wait is bounded and sets the error word instead of hanging.
 // Measured, whole decompositions, update kernel per step -> this: 840 functions
 // (899 steps, 54 passes) 42.3 -> 32.8 ms, 600 (1224 steps) 45.9 -> 30.7 ms, 240 (377
-// steps) 10.4 -> 5.4 ms.  A step of the first takes 14 us: 7 us the column, the
-// rows since the pass and the residuals, 2 us the block maxima, 3 us the exchange.
+// steps) 10.4 -> 5.4 ms; the first 30.9 with the float pairs' conversions in integer
+// operations here and in the digit store.  A step of it takes 13 us: 6 us the column,
+// the rows since the pass and the residuals, 2 us the block maxima, 3 us the exchange.
 #pragma once
 
 namespace cds {
