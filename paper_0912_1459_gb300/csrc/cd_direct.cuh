@@ -39,6 +39,7 @@ constexpr int kDirMaxCtas = 160;            // five lines per lane of a deciding
 constexpr int kDirBoys = (kBoysPoints * kBoysStride + 1) / 2 * 2;   // whole 16-byte units
 constexpr int kDirBits = 26;                // bits of lo
 constexpr int kDirTop = 30;                 // bits of hi
+constexpr int kDirMinExp = -960;
 constexpr int kDirMaxRank = 4096;           // 2 x 2^55 x sqrt(4096) < 2^63
 constexpr size_t kDirSmemMax = 220 * 1024;
 
@@ -161,9 +162,13 @@ k_cd_direct(const __grid_constant__ CdDirectArgs one, const CdDirectArgs* table,
             own[2 * pc] = ok ? a.pd.Py[I] : 0.0;
             own[3 * pc] = ok ? a.pd.Pz[I] : 0.0;
             own[4 * pc] = ok ? a.pd.Kp[I] : 0.0;
-            const double root = sqrt(fmax(dreg[r], 0.0));
+            // sqrt(D0_I), from the pair's factors where D0_I = 2 pi^(5/2) (K/p)^2 / sqrt(2 p)
+            // itself leaves the normal range (pairs of centres far apart, L^K_I of 1e-150 and less)
+            const double root = dreg[r] < 1e-290 ? own[4 * pc] * sqrt(kTwoPi52 * rsqrt(2.0 * own[0]))
+                                                 : sqrt(dreg[r]);
             int e = 0;
             if (root > 0.0 && root < INFINITY) frexp(root, &e);     // root < 2^e
+            e = max(e, kDirMinExp);                                 // 2^(e - 30) stays normal
             own[5 * pc] = ldexp(1.0, e - kDirTop);
             if (ok) a.sc[I] = own[5 * pc];
         }
