@@ -109,6 +109,8 @@ k_cd_direct(const __grid_constant__ CdDirectArgs one, const CdDirectArgs* table,
     __shared__ long long s_wmax[8], s_wmin[8];
     __shared__ uint32_t s_widx[8];
     __shared__ int2 s_new;
+    __shared__ long long s_okey;
+    __shared__ uint32_t s_oidx;
     __shared__ int s_amb, s_fail, s_best;
     __shared__ double s_rdp, s_dp;
     __shared__ long long s_pick;
@@ -257,20 +259,11 @@ k_cd_direct(const __grid_constant__ CdDirectArgs one, const CdDirectArgs* table,
                 if (I == bi) s_new = qv[r];
             }
             if (__any_sync(0xffffffffu, other) && lane == 0) s_amb = 1;
-            named_sync(3, W);
-            if (tid < 32) {
-                const uint32_t ix = (bm >= 0 ? bi : kIdxNone) | (s_amb ? kIdxAmbiguous : 0u);
-                const int2 f = s_new;
-                const long long key = neg ? LLONG_MAX : bm;   // too negative: above every number
-                const uint32_t v = lane == 0   ? (uint32_t)(key >> 32)
-                                   : lane == 1 ? (uint32_t)key
-                                   : lane == 2 ? ix
-                                   : lane == 3 ? (uint32_t)f.x
-                                               : (uint32_t)f.y;
-                if (lane < 5) st_relaxed(words + (size_t)cta * 16 + lane, ((unsigned long long)v << 32) | tag);
-                __syncwarp();
-                if (lane == 0) s_amb = 0;
+            if (tid == 0) {
+                s_okey = neg ? LLONG_MAX : bm;   // too negative: above every number
+                s_oidx = bm >= 0 ? bi : kIdxNone;
             }
+            named_arrive(4, W + 32);             // the deciding warp stores the line
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
                 const int64_t I = base + r * W + tid;
@@ -280,13 +273,22 @@ k_cd_direct(const __grid_constant__ CdDirectArgs one, const CdDirectArgs* table,
                 }
             }
         } else if (decider) {
-            if (lane == 0) {
-                // the last row (at k = 0 the scales) before this step's words
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                s_rdp = 1.0 / sqrt(dp);
-            }
+            // the last row (at k = 0 the scales) before this step's words: fence and words by
+            // the same threads, so a reader that acquires a word sees the rows behind it
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
+            if (lane == 0) s_rdp = 1.0 / sqrt(dp);
             __syncwarp();
             named_arrive(5, W + 32);
+            named_sync(4, W + 32);               // the column group's maximum
+            const int2 f = s_new;
+            const uint32_t v = lane == 0   ? (uint32_t)(s_okey >> 32)
+                               : lane == 1 ? (uint32_t)s_okey
+                               : lane == 2 ? (s_oidx | (s_amb ? kIdxAmbiguous : 0u))
+                               : lane == 3 ? (uint32_t)f.x
+                                           : (uint32_t)f.y;
+            if (lane < 5) st_relaxed(words + (size_t)cta * 16 + lane, ((unsigned long long)v << 32) | tag);
+            __syncwarp();
+            if (lane == 0) s_amb = 0;
         } else {
             const int dt = tid - W;
             if (k > 0) {

@@ -17,9 +17,10 @@
 //    round trip).  A CTA's words are one 128-byte line, written by one store: with
 //    a line shared by several writers the readers' polls took it in turns with
 //    the writes, 7 us a step;
-//  - the fence behind a row (4-6 us when a publisher waited for it) is made by the
-//    deciding warp while the others form the next column, so a row is read by
-//    other CTAs from the step after the next on, and the newest from the words;
+//  - the fence behind a row (4-6 us when the column's warps waited for it) is made by
+//    the deciding warp, which stores the words, while the others form the next column,
+//    so a row is read by other CTAs from the step after the next on, and the newest
+//    from the words;
 //  - every CTA gathers all blocks' words and takes the same decision: stop test,
 //    pivot, candidate slot.  A warp of its own decides, with integer keys, and
 //    forms 1 / sqrt(D_P) while the others form the next column.
@@ -344,43 +345,46 @@ __device__ __forceinline__ void cd_steps_body(const CdStepsArgs& a, int cta, int
                 }
                 if (__any_sync(0xffffffffu, other) && lane == 0) out.amb = 1;
                 if (tt == 0) { out.bm = bm; out.bi = bi; out.neg = neg; }
-                // the CTA's blocks of this turn, one line by one store
+                // the deciding warp stores the line of this turn's blocks
                 const int on_sub = min(nsub, nblk - (r * ncta + cta) * nsub);
-                asm volatile("bar.sync 6, %0;" ::"r"(256 * on_sub) : "memory");
-                if (tid < 32) {
-                    const int q = lane / 5, f = lane - 5 * q;
-                    if (q < on_sub) {
-                        const Block& o = s_out[r & 1][q];
-                        const uint32_t ix = (o.bm >= 0 ? o.bi : kIdxNone) |
-                                            (o.amb ? kIdxAmbiguous : 0u) | (o.neg ? kIdxNegative : 0u);
-                        const uint32_t v = f == 0   ? (uint32_t)(o.bm >> 32)
-                                           : f == 1 ? (uint32_t)o.bm
-                                           : f == 2 ? ix
-                                           : f == 3 ? __float_as_uint(o.fresh.x)
-                                                    : __float_as_uint(o.fresh.y);
-                        st_relaxed(words + (size_t)(r * ncta + cta) * 16 + lane,
-                                   ((unsigned long long)v << 32) | tag);
-                    }
-                    __syncwarp();
-                    if (lane < kStepsMaxSub) s_out[r & 1][lane].amb = 0;
-                }
+                asm volatile("bar.sync 6, %0;" ::"r"(256 * on_sub + 32) : "memory");
 #pragma unroll
                 for (int q = 0; q < kStepPer; ++q) {
                     const int64_t I = base + q * kUpdThreads + tt;
                     if (I < n) Lf[(int64_t)k * n + I] = lf[q];
                 }
             }
-        } else if (k > k0) {   // (the first step's comes with the state)
-            if (lane == 0) {
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");   // the last row before the next words
+        } else {
+            // the last row before this step's words: fence and words by the same threads, so a
+            // reader that acquires a word sees the rows behind it
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
+            if (k > k0 && lane == 0) {   // (the first step's comes with the state)
                 const double rDP = 1.0 / sqrt(s_dp);
                 const float h = (float)rDP;
                 s_rdp = make_float2(h, (float)(rDP - (double)h));
             }
             __syncwarp();
             asm volatile("bar.arrive 5, %0;" ::"r"((int)blockDim.x) : "memory");
-        } else {
-            asm volatile("bar.arrive 5, %0;" ::"r"((int)blockDim.x) : "memory");
+            // the CTA's blocks of each turn, one line by one store
+            for (int r = 0; r < per; ++r) {
+                const int on_sub = min(nsub, nblk - (r * ncta + cta) * nsub);
+                if (on_sub <= 0) break;
+                asm volatile("bar.sync 6, %0;" ::"r"(256 * on_sub + 32) : "memory");
+                const int q = lane / 5, f = lane - 5 * q;
+                if (q < on_sub) {
+                    const Block& o = s_out[r & 1][q];
+                    const uint32_t ix = (o.bm >= 0 ? o.bi : kIdxNone) | (o.amb ? kIdxAmbiguous : 0u) |
+                                        (o.neg ? kIdxNegative : 0u);
+                    const uint32_t v = f == 0   ? (uint32_t)(o.bm >> 32)
+                                       : f == 1 ? (uint32_t)o.bm
+                                       : f == 2 ? ix
+                                       : f == 3 ? __float_as_uint(o.fresh.x)
+                                                : __float_as_uint(o.fresh.y);
+                    st_relaxed(words + (size_t)(r * ncta + cta) * 16 + lane, ((unsigned long long)v << 32) | tag);
+                }
+                __syncwarp();
+                if (lane < kStepsMaxSub) s_out[r & 1][lane].amb = 0;
+            }
         }
         // gather every block's words of this step; each warp keeps its largest key,
         // the block it is in, and whether another of its blocks is in that key's band
