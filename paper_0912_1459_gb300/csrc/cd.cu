@@ -1250,7 +1250,7 @@ static CdLayout cd_layout(void* ws, int32_t nbf, bool spec = true, bool tc = fal
     l.err = direct ? c.take<int32_t>(4) : l.err;
     l.Q = direct ? c.take<int2>((size_t)std::min<int64_t>(max_rank, n) * n) : nullptr;
     l.sc = direct ? c.take<double>(n) : nullptr;
-    l.words = direct ? c.take<unsigned long long>(2 * 16 * kDirMaxCtas) : nullptr;
+    l.words = direct ? dir_words(c.take<unsigned long long>(kDirWordsRoom)) : nullptr;
     l.bytes = c.off;
     return l;
 }
@@ -1609,12 +1609,12 @@ int cd_decompose_run(int32_t nbf, const double* xyz, const double* alpha, const 
             da.cand = dl.cand;
             da.pd = dl.pd;
             da.words[0] = dl.words;
-            da.words[1] = dl.words + 16 * kDirMaxCtas;
+            da.words[1] = dl.words + kDirWords / 2;
             da.piv = piv;
             da.ctrl = dl.ctrl;
             da.err = dl.err;
             CDS_CUDA_TRY(cudaMemsetAsync(dl.err, 0, sizeof(int32_t), stream));
-            CDS_CUDA_TRY(cudaMemsetAsync(dl.words, 0, 2 * 16 * kDirMaxCtas * sizeof(unsigned long long), stream));
+            CDS_CUDA_TRY(cudaMemsetAsync(dl.words, 0, kDirWords * sizeof(unsigned long long), stream));
             da.srows = direct_rows(da.sh, da.kcap);
             if ((st = launch_direct(da, nullptr, 1, da.ctas, direct_smem(da.sh, da.kcap, da.srows), stream)))
                 return st;
@@ -1941,14 +1941,13 @@ static std::vector<DirectWave> direct_waves(int32_t nmol, const BatchMol* mols) 
     }
     return waves;
 }
-constexpr size_t kDirWords = 2 * 16 * (size_t)kDirMaxCtas;
 size_t cd_batch_direct_bytes(int32_t nmol, const BatchMol* mols) {
     const std::vector<DirectWave> waves = direct_waves(nmol, mols);
     size_t rows = 0;
     for (const DirectWave& w : waves) rows = std::max(rows, w.rows_bytes);
     return waves.empty() ? 0
                          : align_up(sizeof(CdDirectArgs) * nmol) + align_up(16) +
-                               align_up(kDirWords * sizeof(unsigned long long)) + align_up(rows);
+                               align_up(kDirWordsRoom * sizeof(unsigned long long)) + align_up(rows);
 }
 static int cd_batch_direct(int32_t nmol, const BatchMol* mols, const std::vector<CdMol>& h,
                            const CdCtrl* ctrl, int32_t* M_out, char* ws, cudaStream_t stream) {
@@ -1956,7 +1955,7 @@ static int cd_batch_direct(int32_t nmol, const BatchMol* mols, const std::vector
     Carver top(ws);
     CdDirectArgs* table = top.take<CdDirectArgs>(nmol);
     int32_t* err = top.take<int32_t>(4);
-    unsigned long long* words = top.take<unsigned long long>(kDirWords);
+    unsigned long long* words = dir_words(top.take<unsigned long long>(kDirWordsRoom));
     char* rows = top.take<char>(0);
     std::vector<CdDirectArgs> ha;
     for (const DirectWave& w : waves) {

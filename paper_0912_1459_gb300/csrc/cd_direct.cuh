@@ -76,6 +76,14 @@ struct CdDirectArgs {
     int32_t* err;
 };
 
+// The words of one launch: two sets of a 128-byte line per CTA, on lines of their own
+// (they are read 16 bytes at a time) whatever the caller's workspace starts at.
+constexpr size_t kDirWords = 2 * 16 * (size_t)kDirMaxCtas;
+constexpr size_t kDirWordsRoom = kDirWords + 16;
+inline unsigned long long* dir_words(unsigned long long* room) {
+    return reinterpret_cast<unsigned long long*>(align_up((size_t)room, 128));
+}
+
 __host__ __device__ inline size_t direct_smem(const DirectShape& s, int32_t kcap, int32_t srows) {
     return (size_t)kDirBoys * 8 + (size_t)(kcap + 1) / 2 * 2 * 8 + (size_t)s.groups * s.pc * 16 +
            (size_t)s.pc * 6 * 8 + (size_t)srows * s.pc * 8;
