@@ -54,7 +54,11 @@ typedef enum {
 typedef enum { CDS_SCHEME_FULL = 0, CDS_SCHEME_ATOMIC = 1 } cds_scheme;
 
 /* Arithmetic of the J-contractions in sigma2 / qp_solve.
- * FP64: binary64 throughout (CUDA cores).
+ * FP64: binary64 inputs, sums and results.  A product sum_K a_K b_K is good to
+ *   M 2^-53 sum_K |a_K||b_K|, as a sum of M FP64 products is, whatever the range
+ *   of the rows; from 64 orbitals on (transform: 32 functions) the products are
+ *   formed from exact eight-digit slices on the tensor cores, and those whose sum
+ *   of magnitudes is below 2^-5 of the rows' scales on the FP64 units.
  * BF16X3 / FP16X3 / TF32X3: each factor split s*x = hi + lo with hi, lo bf16
  *   (s = 1), fp16 (s = a power of two with max|s x| <= 1024) or tf32 (s = 1,
  *   FP32 containers); the products hi*hi + hi*lo + lo*hi run on tcgen05

@@ -23,8 +23,7 @@ namespace cds {
 int launch_dgemm_strided(int m, int n, int k, int batch, const double* A, int64_t ars, int64_t acs,
                          int64_t abs_, const double* B, int64_t brs, int64_t bcs, int64_t bbs,
                          double* C, int64_t crs, int64_t ccs, int64_t cbs, cudaStream_t s,
-                         bool accumulate = false,
-                         const int32_t* only_if = nullptr);
+                         bool accumulate = false);
 void make_terms(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* Lp,
                 const double* eps, SigmaTerm& t0, SigmaTerm& t1);
 

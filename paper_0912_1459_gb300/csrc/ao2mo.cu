@@ -50,12 +50,9 @@ struct StridedOut {
 
 // C[b] (m x n) = A[b] (m x k) * B[b] (k x n), all operands by strides.
 // A_M_CONTIG: A's unit stride is along m; B_N_CONTIG: B's unit stride is along n.
-// only_if (may be null): a device flag; the launch returns at once while it is 0.
 template <bool A_M_CONTIG, bool B_N_CONTIG, bool ACC = false>
 __global__ void __launch_bounds__(256)
-k_dgemm(int m, int n, int k, StridedMat A, StridedMat B, StridedOut C,
-        const int32_t* __restrict__ only_if) {
-    if (only_if && *only_if == 0) return;
+k_dgemm(int m, int n, int k, StridedMat A, StridedMat B, StridedOut C) {
     __shared__ double As[kGK][kGB + 1];
     __shared__ double Bs[kGK][kGB + 1];
     const int tid = threadIdx.x;
@@ -326,34 +323,34 @@ __global__ void k_gather_cols(const double* __restrict__ C, int32_t N, int32_t n
 
 template <bool AM, bool BN, bool ACC = false>
 static int launch_dgemm(int m, int n, int k, int batch, StridedMat A, StridedMat B, StridedOut C,
-                        cudaStream_t s, const int32_t* only_if = nullptr) {
+                        cudaStream_t s) {
     if (m <= 0 || n <= 0 || batch <= 0) return CDS_OK;
     dim3 grid((n + kGB - 1) / kGB, (m + kGB - 1) / kGB, batch);
-    k_dgemm<AM, BN, ACC><<<grid, 256, 0, s>>>(m, n, k, A, B, C, only_if);
+    k_dgemm<AM, BN, ACC><<<grid, 256, 0, s>>>(m, n, k, A, B, C);
     CDS_LAUNCH_CHECK();
     return CDS_OK;
 }
 
 // Strided-batched FP64 GEMM for other translation units; picks the load
 // pattern from the unit strides.  accumulate: C += A B (batch entries must
-// then write disjoint C).  only_if: as k_dgemm.
+// then write disjoint C).
 int launch_dgemm_strided(int m, int n, int k, int batch, const double* A, int64_t ars, int64_t acs,
                          int64_t abs_, const double* B, int64_t brs, int64_t bcs, int64_t bbs,
                          double* C, int64_t crs, int64_t ccs, int64_t cbs, cudaStream_t s,
-                         bool accumulate = false, const int32_t* only_if = nullptr) {
+                         bool accumulate = false) {
     StridedMat Am{A, ars, acs, abs_}, Bm{B, brs, bcs, bbs};
     StridedOut Cm{C, crs, ccs, cbs};
     const bool am = ars == 1, bn = bcs == 1;
     if (accumulate) {
-        if (am && bn) return launch_dgemm<true, true, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
-        if (am) return launch_dgemm<true, false, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
-        if (bn) return launch_dgemm<false, true, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
-        return launch_dgemm<false, false, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+        if (am && bn) return launch_dgemm<true, true, true>(m, n, k, batch, Am, Bm, Cm, s);
+        if (am) return launch_dgemm<true, false, true>(m, n, k, batch, Am, Bm, Cm, s);
+        if (bn) return launch_dgemm<false, true, true>(m, n, k, batch, Am, Bm, Cm, s);
+        return launch_dgemm<false, false, true>(m, n, k, batch, Am, Bm, Cm, s);
     }
-    if (am && bn) return launch_dgemm<true, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
-    if (am) return launch_dgemm<true, false>(m, n, k, batch, Am, Bm, Cm, s, only_if);
-    if (bn) return launch_dgemm<false, true>(m, n, k, batch, Am, Bm, Cm, s, only_if);
-    return launch_dgemm<false, false>(m, n, k, batch, Am, Bm, Cm, s, only_if);
+    if (am && bn) return launch_dgemm<true, true>(m, n, k, batch, Am, Bm, Cm, s);
+    if (am) return launch_dgemm<true, false>(m, n, k, batch, Am, Bm, Cm, s);
+    if (bn) return launch_dgemm<false, true>(m, n, k, batch, Am, Bm, Cm, s);
+    return launch_dgemm<false, false>(m, n, k, batch, Am, Bm, Cm, s);
 }
 
 // U2[mu][b][nu] = L[K0+b][pair(mu,nu)] (vector index inside the row, so the
@@ -503,8 +500,7 @@ template <int RM>
 __global__ void __launch_bounds__(256)
 k_dchain(const double* __restrict__ L, int64_t npair, int32_t N, int32_t K0, int32_t kb,
          const double* __restrict__ C, int32_t nmo, int32_t nocc, const int32_t* __restrict__ orb,
-         int32_t r_first, int32_t r_end, double* __restrict__ T, const int32_t* __restrict__ only_if) {
-    if (only_if && *only_if == 0) return;
+         int32_t r_first, int32_t r_end, double* __restrict__ T) {
     constexpr int R = 4 * RM;
     __shared__ double As[kGK][R];
     __shared__ double Bs[kGK][64];
@@ -553,7 +549,7 @@ k_dchain(const double* __restrict__ L, int64_t npair, int32_t N, int32_t K0, int
 // Rows [r_first, r_end) of T in blocks of at most 64 rows, as even as they go.
 static int dchain(const double* L, int32_t N, int32_t K0, int32_t kb, const double* C, int32_t nmo,
                   int32_t nocc, const int32_t* orb, int32_t r_first, int32_t r_end, double* T,
-                  const int32_t* only_if, cudaStream_t stream) {
+                  cudaStream_t stream) {
     const int rows = r_end - r_first;
     if (rows <= 0 || kb <= 0) return CDS_OK;
     const int nb = (rows + 63) / 64, rm = ((rows + nb - 1) / nb + 7) / 8 * 2;
@@ -561,7 +557,7 @@ static int dchain(const double* L, int32_t N, int32_t K0, int32_t kb, const doub
 #define CDS_DCHAIN(RM_)                                                                          \
     case RM_:                                                                                    \
         k_dchain<RM_><<<grid, 256, 0, stream>>>(L, npair_of(N), N, K0, kb, C, nmo, nocc, orb,    \
-                                                r_first, r_end, T, only_if);                     \
+                                                r_first, r_end, T);                              \
         break
     switch (rm) {
         CDS_DCHAIN(2);
@@ -582,20 +578,19 @@ static int dchain(const double* L, int32_t N, int32_t K0, int32_t kb, const doub
 // Lov[i][a][K0 + b] and Lp[t][r][K0 + b] from T on the FP64 units.
 static int fp64_second(int32_t N, int32_t nmo, int32_t nocc, int32_t np, const double* C, int32_t K0,
                        int32_t kb, int32_t M, const double* T, double* Lov, double* Lp,
-                       const int32_t* only_if, cudaStream_t stream) {
+                       cudaStream_t stream) {
     const int32_t nv = nmo - nocc;
     const int64_t trow = (int64_t)kb * N;
     if (nocc > 0 && nv > 0) {
         const int st = launch_dgemm<false, true>(
             nocc, nv, N, kb, StridedMat{T, trow, 1, N}, StridedMat{C + nocc, nmo, 1, 0},
-            StridedOut{Lov + K0, (int64_t)nv * M, M, 1}, stream, only_if);
+            StridedOut{Lov + K0, (int64_t)nv * M, M, 1}, stream);
         if (st) return st;
     }
     if (np > 0)
         return launch_dgemm<false, true>(np, nmo, N, kb, StridedMat{T + nocc * trow, trow, 1, N},
                                          StridedMat{C, nmo, 1, 0},
-                                         StridedOut{Lp + K0, (int64_t)nmo * M, M, 1}, stream,
-                                         only_if);
+                                         StridedOut{Lp + K0, (int64_t)nmo * M, M, 1}, stream);
     return CDS_OK;
 }
 
@@ -619,7 +614,7 @@ struct DxLayout {
     dx::Operand cj, cv, ca;   // columns of C: occupied | requested, virtual, all
     dx::Operand u, tov, tp;   // rows (K, nu) of the vectors, rows (i, K) and (t, K) of T
     double* T;                // [(r, K)][nu]
-    int32_t* flag;            // [0] an operand is not finite, [1] error word
+    int32_t* err;             // error word
     size_t bytes;
 };
 
@@ -636,7 +631,7 @@ static DxLayout dx_layout(void* ws, int32_t N, int32_t nmo, int32_t nocc, int32_
     l.tov = dx::carve(c, 1, (int64_t)kb * nocc, N, dx::kRowsA);
     l.tp = dx::carve(c, 1, (int64_t)kb * np, N, dx::kRowsA);
     l.T = c.take<double>((size_t)std::max(nocc + np, 1) * kb * N);
-    l.flag = c.take<int32_t>(2);
+    l.err = c.take<int32_t>(1);
     l.bytes = c.off + 256;
     return l;
 }
@@ -655,22 +650,16 @@ static int cd_to_mo_fp64(int32_t N, int32_t nmo, int32_t nocc, int32_t M, const 
     if (dx_serves(N, nmo, nocc, np) && ws_bytes >= dx_layout(nullptr, N, nmo, nocc, np, kbx).bytes) {
         const DxLayout l = dx_layout(ws, N, nmo, nocc, np, kbx);
         const bool ov = nocc > 0 && nv > 0;
-        int32_t *flag = l.flag, *err = l.flag + 1;
-        CDS_CUDA_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(int32_t), stream));
+        CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
         if (!ov && np == 0) return CDS_OK;
         const bool chain = N <= kDxChainBasis;
         const int32_t r0 = ov ? 0 : nocc;   // the occupied rows only when Lov is wanted
+        const dx::Columns cj{C, orb, nmo, nocc, 0}, cv{C, nullptr, nmo, nmo, nocc}, ca{C, nullptr, nmo, nmo, 0};
         int st = CDS_OK;
-        if (!chain)
-            st = dx::slice_columns(dx::Columns{C, orb, nmo, nocc, 0}, l.cj, dx::kRowsB, N, flag, stream);
-        if (!st && ov)
-            st = dx::slice_columns(dx::Columns{C, nullptr, nmo, nmo, nocc}, l.cv, dx::kRowsB, N, flag,
-                                   stream);
-        if (!st && np > 0)
-            st = dx::slice_columns(dx::Columns{C, nullptr, nmo, nmo, 0}, l.ca, dx::kRowsB, N, flag,
-                                   stream);
+        if (!chain) st = dx::slice(cj, l.cj, dx::kRowsB, N, stream);
+        if (!st && ov) st = dx::slice(cv, l.cv, dx::kRowsB, N, stream);
+        if (!st && np > 0) st = dx::slice(ca, l.ca, dx::kRowsB, N, stream);
         if (st) return st;
-        const int64_t nocut = INT64_MAX;
         for (int32_t K0 = 0; K0 < M; K0 += kbx) {
             const int32_t kb = std::min(kbx, M - K0);
             auto sized = [](dx::Operand o, int64_t rows, int R) {
@@ -681,44 +670,37 @@ static int cd_to_mo_fp64(int32_t N, int32_t nmo, int32_t nocc, int32_t M, const 
             const dx::Operand tov = sized(l.tov, (int64_t)kb * nocc, dx::kRowsA);
             const dx::Operand tp = sized(l.tp, (int64_t)kb * np, dx::kRowsA);
             const int64_t trow = (int64_t)kb * N;   // elements of T per r
-            if (!chain) {
+            if (chain) {
+                st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, l.T, stream);
+            } else {
                 const dx::Operand u = sized(l.u, (int64_t)kb * N, dx::kRowsA);
-                st = dx::slice_packed(dx::PackedRows{L, npair_of(N), K0, N}, u, dx::kRowsA, N, flag,
-                                      stream);
+                const dx::PackedRows rows{L, npair_of(N), K0, N};
+                st = dx::slice(rows, u, dx::kRowsA, N, stream);
                 if (!st)
-                    st = dx::gemm(u, l.cj, 0, 1, dx::Out{l.T, nocut, 0, 1, 0, trow}, nullptr, flag, err,
-                                  stream);
+                    st = dx::gemm(u, rows, l.cj, cj, N, 0, 1, dx::Out{l.T, INT64_MAX, 0, 1, 0, trow}, nullptr,
+                                  l.err, stream);
             }
-            // the FMA chain: always for the small bases, else for flagged operands
-            if (!st)
-                st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, l.T,
-                            chain ? nullptr : flag, stream);
+            const dx::RowMajor rov{l.T, 0, N}, rp{l.T + nocc * trow, 0, N};
+            if (!st && ov) st = dx::slice(rov, tov, dx::kRowsA, N, stream);
+            if (!st && np > 0) st = dx::slice(rp, tp, dx::kRowsA, N, stream);
             if (!st && ov)
-                st = dx::slice_rows(dx::RowMajor{l.T, 0, N}, tov, dx::kRowsA, N, flag, stream);
+                st = dx::gemm(tov, rov, l.cv, cv, N, 0, 1, dx::Out{Lov + K0, kb, (int64_t)nv * M, 1, 0, M},
+                              nullptr, l.err, stream);
             if (!st && np > 0)
-                st = dx::slice_rows(dx::RowMajor{l.T + nocc * trow, 0, N}, tp, dx::kRowsA, N, flag,
-                                    stream);
-            if (!st && ov)
-                st = dx::gemm(tov, l.cv, 0, 1,
-                              dx::Out{Lov + K0, kb, (int64_t)nv * M, 1, 0, M}, nullptr, flag, err,
-                              stream);
-            if (!st && np > 0)
-                st = dx::gemm(tp, l.ca, 0, 1, dx::Out{Lp + K0, kb, (int64_t)nmo * M, 1, 0, M}, nullptr,
-                              flag, err, stream);
-            if (!st)
-                st = fp64_second(N, nmo, nocc, np, C, K0, kb, M, l.T, Lov, Lp, flag, stream);
+                st = dx::gemm(tp, rp, l.ca, ca, N, 0, 1, dx::Out{Lp + K0, kb, (int64_t)nmo * M, 1, 0, M},
+                              nullptr, l.err, stream);
             if (st) return st;
         }
-        if (ov && (st = dx::nan_on_error(err, Lov, (int64_t)nocc * nv * M, stream))) return st;
-        if (np > 0 && (st = dx::nan_on_error(err, Lp, (int64_t)np * nmo * M, stream))) return st;
+        if (ov && (st = dx::nan_on_error(l.err, Lov, (int64_t)nocc * nv * M, stream))) return st;
+        if (np > 0 && (st = dx::nan_on_error(l.err, Lp, (int64_t)np * nmo * M, stream))) return st;
         return CDS_OK;
     }
     const AoLayout lay = ao_layout(ws, N, nmo, nocc, np);
     const int32_t r0 = nocc > 0 && nv > 0 ? 0 : nocc;
     for (int32_t K0 = 0; K0 < M; K0 += kAoBatch) {
         const int32_t kb = std::min(kAoBatch, M - K0);
-        int st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, lay.T, nullptr, stream);
-        if (!st) st = fp64_second(N, nmo, nocc, np, C, K0, kb, M, lay.T, Lov, Lp, nullptr, stream);
+        int st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, lay.T, stream);
+        if (!st) st = fp64_second(N, nmo, nocc, np, C, K0, kb, M, lay.T, Lov, Lp, stream);
         if (st) return st;
     }
     return CDS_OK;

@@ -3,10 +3,20 @@
 // B[n][k] from operands stored as eight signed base-256 digits per element.
 //
 // A row is scaled by 2^ex > max|x| of the row, q = round(x 2^(62-ex)) (exact
-// for every entry within 2^-9 of the row's largest, 2^-63 of it otherwise),
-// and q is cut into eight digits d_0 (most significant, |d_0| <= 64) .. d_7
-// in [-128, 127], each exact in BF16.  The 36 digit products with s + t <= 7
-// are kept; the dropped ones are below 2^-60 of both rows' scales.
+// for every entry within 2^-9 of the row's largest, to 2^-63 of the scale
+// otherwise), and q is cut into eight digits d_0 (most significant, |d_0| <= 64)
+// .. d_7 in [-128, 127], each exact in BF16.  The 36 digit products with s + t <= 7
+// are kept.  In units of both rows' scales the result of K columns is off by at most
+// K 2^-58.9: 7 x 2^14 x 2^-76 a column from the dropped products with s + t = 8, 2^-62
+// from the rounding of q, 2^-61 from FP32 sums beyond 2^24 (weights 6 and 7 of columns
+// whose low digits agree).  Digits of unrelated numbers leave sqrt(K) 2^-62.
+//
+// That is a bound on the rows' scales, where a sum of FP64 products is good to K 2^-53
+// S, S = sum_k |a_k||b_k|, however small S is beside them.  So a second pass forms S,
+// from the magnitudes of the operands in BF16 (rounded down), and takes the results
+// with S < 2^-5 of the scales again, each as an FP64 sum over the rows themselves:
+// every result is good to K 2^-53 S.  Rows that are not finite, or beyond 2^+-400, have
+// magnitudes of zero and are all taken so.
 #pragma once
 
 #include "common.cuh"
@@ -21,10 +31,11 @@ constexpr int kDigits = 8;
 
 // One sliced operand: tiles of R rows, each [k-step][digit][R rows x 32
 // bytes], already in the order and 32-byte swizzle the MMA reads, so a k-step
-// of a tile is one contiguous bulk copy.  Rows come in groups of `per` that
-// start on a tile boundary (per = all rows for a plain matrix).
+// of a tile is one contiguous bulk copy; mag the same with |x| / 2^ex in place of
+// the digits.  Rows come in groups of `per` that start on a tile boundary (per =
+// all rows for a plain matrix).
 struct Operand {
-    uint8_t* img;
+    uint8_t *img, *mag;
     int32_t* ex;       // scale exponent per padded row
     int64_t groups, per, per_pad;
     int32_t ksteps;
@@ -39,59 +50,77 @@ inline Operand carve(Carver& c, int64_t groups, int64_t per, int32_t kdim, int R
     o.ksteps = ksteps_of(kdim);
     const size_t rows = (size_t)(groups * o.per_pad);
     o.img = c.take<uint8_t>(rows * o.ksteps * kDigits * kStepK * 2);
+    o.mag = c.take<uint8_t>(rows * o.ksteps * kStepK * 2);
     o.ex = c.take<int32_t>(rows);
     return o;
 }
 
-// Row sources: element k of row r of group g.
+// Row sources: row(g, r)[k] is element k of row r of group g.  kAcross: neighbouring
+// rows, not neighbouring k, lie side by side in memory.
 struct RowMajor {         // x[(g gs + r) ld + k]
+    static constexpr bool kAcross = false;
     const double* x;
     int64_t gs, ld;
-    __device__ __forceinline__ double get(int64_t g, int64_t r, int k) const {
-        return x[(g * gs + r) * ld + k];
-    }
+    struct Row {
+        const double* x;
+        __device__ __forceinline__ double operator[](int k) const { return x[k]; }
+    };
+    __device__ __forceinline__ Row row(int64_t g, int64_t r) const { return {x + (g * gs + r) * ld}; }
 };
 struct PackedRows {       // rows (K, nu): A^K[nu][k] of the packed symmetric vectors
+    static constexpr bool kAcross = false;
     const double* L;
     int64_t npair;
     int32_t K0, N;
-    __device__ __forceinline__ double get(int64_t, int64_t r, int k) const {
-        const int K = (int)(r / N), nu = (int)(r % N);
-        const int hi = max(k, nu), lo = min(k, nu);
-        return L[(int64_t)(K0 + K) * npair + (int64_t)hi * (hi + 1) / 2 + lo];
+    struct Row {
+        const double* L;
+        int nu;
+        __device__ __forceinline__ double operator[](int k) const {
+            const int hi = max(k, nu), lo = min(k, nu);
+            return L[(int64_t)hi * (hi + 1) / 2 + lo];
+        }
+    };
+    __device__ __forceinline__ Row row(int64_t, int64_t r) const {
+        return {L + (int64_t)(K0 + (int)(r / N)) * npair, (int)(r % N)};
     }
 };
 struct Columns {          // row j: C[k][col(j)], col(j) = j < nocc ? j : orb[j - nocc]
+    static constexpr bool kAcross = true;
     const double* C;
     const int32_t* orb;
     int32_t nmo, nocc, first;
-    __device__ __forceinline__ double get(int64_t, int64_t r, int k) const {
+    struct Row {
+        const double* C;      // null: no such orbital, NaN
+        int64_t ld;
+        __device__ __forceinline__ double operator[](int k) const {
+            return C ? C[k * ld] : __longlong_as_double(0x7ff8000000000000LL);
+        }
+    };
+    __device__ __forceinline__ Row row(int64_t, int64_t r) const {
         int q = (int)r + first;
         if (orb && q >= nocc) q = orb[q - nocc];
-        if (q < 0 || q >= nmo) return __longlong_as_double(0x7ff8000000000000LL);
-        return C[(int64_t)k * nmo + q];
+        return {q >= 0 && q < nmo ? C + q : nullptr, nmo};
     }
 };
 
-// Slice an operand (R = kRowsA or kRowsB).  *flag is set (never cleared) when
-// a row holds a non-finite entry or a magnitude outside 2^+-400: the products
-// of such a call are then left to the plain FP64 kernel (run_gemm's fallback).
-int slice_rows(const RowMajor& src, const Operand& o, int R, int32_t kdim, int32_t* flag,
-               cudaStream_t stream);
-int slice_packed(const PackedRows& src, const Operand& o, int R, int32_t kdim, int32_t* flag,
-                 cudaStream_t stream);
-int slice_columns(const Columns& src, const Operand& o, int R, int32_t kdim, int32_t* flag,
-                  cudaStream_t stream);
+// Slice an operand (R = kRowsA or kRowsB).
+int slice(const RowMajor& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
+int slice(const PackedRows& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
+int slice(const Columns& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
 
 // out[(m / kdiv) m_hi + (m % kdiv) m_lo + (g - g0) g_s + n n_s] for the rows m of
 // A (one group) and the rows n < B.per of B's groups [g0, g1).  Groups whose
-// active[g] is 0 are skipped.  Returns at once on the device when *flag is set.
+// active[g] is 0 are skipped.  a, b: the sources that A and B were sliced from.
 struct Out {
     double* p;
     int64_t kdiv, m_hi, m_lo, g_s, n_s;
 };
-int gemm(const Operand& A, const Operand& B, int64_t g0, int64_t g1, const Out& out,
-         const int32_t* active, const int32_t* flag, int32_t* err, cudaStream_t stream);
+int gemm(const Operand& A, const RowMajor& a, const Operand& B, const RowMajor& b, int32_t kdim, int64_t g0,
+         int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream);
+int gemm(const Operand& A, const PackedRows& a, const Operand& B, const Columns& b, int32_t kdim, int64_t g0,
+         int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream);
+int gemm(const Operand& A, const RowMajor& a, const Operand& B, const Columns& b, int32_t kdim, int64_t g0,
+         int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream);
 
 // p[0..n) = NaN when *err is set (a device-side wait gave up).
 int nan_on_error(const int32_t* err, double* p, int64_t n, cudaStream_t stream);

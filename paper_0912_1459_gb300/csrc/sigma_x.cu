@@ -23,11 +23,6 @@
 
 namespace cds {
 
-int launch_dgemm_strided(int m, int n, int k, int batch, const double* A, int64_t ars, int64_t acs,
-                         int64_t abs_, const double* B, int64_t brs, int64_t bcs, int64_t bbs,
-                         double* C, int64_t crs, int64_t ccs, int64_t cbs, cudaStream_t s,
-                         bool accumulate, const int32_t* only_if);
-
 namespace sx {
 
 constexpr int TB = 32;                      // pair-index block, as k_sigma_fp64
@@ -464,7 +459,7 @@ static int final_sum(const XArgs& a, int32_t np, int32_t nblk, const int32_t* er
 struct Layout {
     dx::Operand ov, p;
     double *X, *part;
-    int32_t* flag;   // [0]: an operand needs the plain FP64 product; [1]: error word
+    int32_t* err;    // error word
     int32_t group, nblk;
     size_t bytes;
 };
@@ -483,21 +478,17 @@ static Layout layout(void* ws, int32_t nmo, int32_t nocc, int32_t M, int32_t np,
     l.X = c.take<double>((size_t)l.group * rows * ov);
     const size_t nz = nE > kDirect ? (size_t)(nE + kZone - 1) / kZone : 1;
     l.part = c.take<double>((size_t)np * nz * l.nblk * part_stride(nE));
-    l.flag = c.take<int32_t>(2);
+    l.err = c.take<int32_t>(1);
     l.bytes = c.off + 256;
     return l;
 }
 
-// X of orbitals [t0, t0 + n), FP64 rows as the plain product when flagged.
+// X of orbitals [t0, t0 + n).
 static int integrals(const Layout& l, int64_t ov, int32_t rows, int32_t M, const double* Lov,
                      const double* Q, int32_t t0, int32_t n, const int32_t* active,
                      cudaStream_t stream) {
-    const dx::Out out{l.X, INT64_MAX, 0, 1, (int64_t)rows * ov, ov};
-    int st = dx::gemm(l.ov, l.p, t0, t0 + n, out, active, l.flag, l.flag + 1, stream);
-    if (st) return st;
-    return launch_dgemm_strided((int)ov, rows, M, n, Lov, M, 1, 0, Q + (int64_t)t0 * rows * M, 1, M,
-                                (int64_t)rows * M, l.X, 1, ov, (int64_t)rows * ov, stream, false,
-                                l.flag);
+    return dx::gemm(l.ov, dx::RowMajor{Lov, 0, M}, l.p, dx::RowMajor{Q, rows, M}, M, t0, t0 + n,
+                    dx::Out{l.X, INT64_MAX, 0, 1, (int64_t)rows * ov, ov}, active, l.err, stream);
 }
 
 }  // namespace sx
@@ -506,8 +497,8 @@ using namespace sx;
 
 bool sigma_x_serves(int32_t nmo, int32_t nocc, int32_t np) {
     const int64_t nv = nmo - nocc, ov = nocc * nv;
-    // grid limits of the plain product; 32-bit item indices per orbital
-    return nmo >= 64 && nocc > 0 && nv > 0 && np > 0 && ov < (1 << 22) && nmo <= (1 << 14) &&
+    // 32-bit item indices per orbital; orbitals in grid.y
+    return nmo >= 64 && nocc > 0 && nv > 0 && np > 0 && np <= 65535 && ov < (1 << 22) && nmo <= (1 << 14) &&
            tc::device_ok();
 }
 
@@ -526,10 +517,10 @@ int sigma2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const doub
     const Layout l = layout(ws, nmo, nocc, M, np, nE, nmo, a.tm[0].per + a.tm[1].per);
     int st = CDS_OK;
     if (resplit) {
-        CDS_CUDA_TRY(cudaMemsetAsync(l.flag, 0, 2 * sizeof(int32_t), stream));
-        if ((st = dx::slice_rows(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, l.flag, stream)))
+        CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
+        if ((st = dx::slice(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, stream)))
             return st;
-        if ((st = dx::slice_rows(dx::RowMajor{Lp, nmo, M}, l.p, dx::kRowsB, M, l.flag, stream)))
+        if ((st = dx::slice(dx::RowMajor{Lp, nmo, M}, l.p, dx::kRowsB, M, stream)))
             return st;
     }
     a.X = l.X;
@@ -547,7 +538,7 @@ int sigma2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const doub
         a.t0 = t0;
         if ((st = eval(a, n, l.nblk, false, stream))) return st;
     }
-    return final_sum(a, np, l.nblk, l.flag + 1, sigma, dsigma, stream);
+    return final_sum(a, np, l.nblk, l.err, sigma, dsigma, stream);
 }
 
 size_t sigma_x_cached_bytes(int32_t nmo, int32_t nocc, int32_t np) {
@@ -595,10 +586,10 @@ int mp2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double*
     XArgs a{};
     mp2_terms(a, nmo, nocc, eps);
     const Layout l = layout(ws, nmo, nocc, M, nocc, 1, nv, a.tm[1].per);
-    CDS_CUDA_TRY(cudaMemsetAsync(l.flag, 0, 2 * sizeof(int32_t), stream));
-    int st = dx::slice_rows(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, l.flag, stream);
+    CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
+    int st = dx::slice(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, stream);
     if (st) return st;
-    if ((st = dx::slice_rows(dx::RowMajor{Lov, nv, M}, l.p, dx::kRowsB, M, l.flag, stream)))
+    if ((st = dx::slice(dx::RowMajor{Lov, nv, M}, l.p, dx::kRowsB, M, stream)))
         return st;
     a.X = l.X;
     a.tstride = (int64_t)nv * ov;
@@ -612,7 +603,7 @@ int mp2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double*
         a.t0 = t0;
         if ((st = eval(a, n, l.nblk, false, stream))) return st;
     }
-    return final_sum(a, nocc, l.nblk, l.flag + 1, e_pair, nullptr, stream);
+    return final_sum(a, nocc, l.nblk, l.err, e_pair, nullptr, stream);
 }
 
 }  // namespace cds
