@@ -378,10 +378,15 @@ int cds_cd_decompose_to_mo(int32_t nbf, const double* xyz, const double* alpha,
  * Diagonal second-order self-energy (paper Eq. SE) and its energy derivative
  * for np orbitals orb[t] at nE energies each:
  *   sigma[t][e]  = Sigma_qq(E[t][e]),  dsigma[t][e] = dSigma_qq/dE (analytic),
- * MO integrals recomputed tile by tile from the factors and never stored.
+ * MO integrals recomputed from the factors at every call.  The split precisions
+ * never store them; FP64 from 64 orbitals on holds those of a group of orbitals, or
+ * of a panel of one orbital's, in the workspace while it sums them.
  * Inputs are the outputs of cds_cd_to_mo plus eps (device [nmo]).
  * ---------------------------------------------------------------------- */
 
+/* FP64 asks for at most 4 GB wherever a panel fits those, and works in less: in narrower
+ * panels, below that in the fused kernel (two doubles per 32 x 32 elements and energy),
+ * which forms the integrals on the FP64 units. */
 size_t cds_sigma2_workspace_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np,
                                   int32_t nE, int32_t precision);
 
@@ -490,7 +495,7 @@ int cds_qp_solve_bracketed_cached(int32_t nmo, int32_t nocc, int32_t np, const i
  * MP2 correlation energy (paper Eq. MP2), the ground-state companion of
  * Eq. SE on the same factors:
  *   E = sum_{i,j,a,b} (2 (ai|bj) - (aj|bi)) (ai|bj) / (e_i + e_j - e_a - e_b),
- *   (ai|bj) = sum_K Lov[i][a][K] Lov[j][b][K], recomputed tile by tile.
+ *   (ai|bj) = sum_K Lov[i][a][K] Lov[j][b][K], formed as for the self-energy.
  * For each i the sum over j, a, b is the second sum of Eq. SE with q := i at
  * E = e_i, and the call runs on the self-energy kernels (FP64, or the
  * tensor-core split precisions).

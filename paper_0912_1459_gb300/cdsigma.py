@@ -177,6 +177,21 @@ def _workspace(nbytes: int, device: torch.device) -> torch.Tensor:
     return torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device=device)
 
 
+def _scratch(need: int, given: Optional[torch.Tensor], device: torch.device,
+             smaller: bool) -> torch.Tensor:
+    """The caller's workspace if it is as large as the call asks for, else one that is.
+    smaller: the call also works in less (FP64 forms), so where the device has no room
+    for what it asks for, the caller's is tried."""
+    if given is not None and given.numel() >= need:
+        return given
+    try:
+        return _workspace(need, device)
+    except torch.OutOfMemoryError:
+        if given is None or not smaller:
+            raise
+        return given
+
+
 def npair(nbf: int) -> int:
     return nbf * (nbf + 1) // 2
 
@@ -243,8 +258,7 @@ def cds_cd_decompose(xyz: torch.Tensor, alpha: torch.Tensor, atom: torch.Tensor,
     piv = torch.empty(max(max_rank, 1), dtype=torch.int32, device=dev)
     D = torch.empty(npr, dtype=torch.float64, device=dev)
     need = lib.cds_cd_workspace_bytes_prec(n, int(max_rank), PRECISIONS[precision])
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     M = _i32(0)
     de = _f64(0.0)
     st = lib.cds_cd_decompose(n, _p(xyz), _p(alpha), _p(atom), float(delta), SCHEMES[scheme],
@@ -468,8 +482,7 @@ def cds_cd_to_mo(L: torch.Tensor, C: torch.Tensor, nocc: int, orbitals: torch.Te
     Lov = torch.empty((nocc, nmo - nocc, M), dtype=torch.float64, device=dev)
     Lp = torch.empty((np_, nmo, M), dtype=torch.float64, device=dev)
     need = lib.cds_cd_to_mo_workspace_bytes(nbf, nmo, nocc, M, np_)
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     _check(lib.cds_cd_to_mo(nbf, nmo, nocc, M, _p(L), _p(C), _p(orb), np_, PRECISIONS[precision],
                             _p(Lov), _p(Lp), _p(workspace), workspace.numel(), _stream(dev)),
            "cds_cd_to_mo")
@@ -494,8 +507,7 @@ def cds_sigma2_diag(Lov: torch.Tensor, Lp: torch.Tensor, eps: torch.Tensor, nocc
     sig = torch.empty((np_, nE), dtype=torch.float64, device=dev)
     dsig = torch.empty((np_, nE), dtype=torch.float64, device=dev)
     need = lib.cds_sigma2_workspace_bytes(nmo, nocc, M, np_, nE, prec)
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     _check(lib.cds_sigma2_diag(nmo, nocc, M, _p(Lov), _p(Lp), np_, _p(eps), _p(E), nE, prec,
                                _p(sig), _p(dsig), _p(workspace), workspace.numel(),
                                _stream(dev)), "cds_sigma2_diag")
@@ -521,8 +533,7 @@ def cds_qp_solve(Lov: torch.Tensor, Lp: torch.Tensor, orbitals: torch.Tensor, ep
     iters = torch.empty(np_, dtype=torch.int32, device=dev)
     status = torch.empty(np_, dtype=torch.int32, device=dev)
     need = lib.cds_qp_workspace_bytes(nmo, nocc, M, np_, prec)
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     st = lib.cds_qp_solve(nmo, nocc, M, _p(Lov), _p(Lp), _p(orb), np_, _p(eps), float(conv),
                           int(max_iter), prec, _p(omega), _p(pole), _p(iters), _p(status),
                           _p(workspace), workspace.numel(), _stream(dev))
@@ -552,8 +563,7 @@ def cds_qp_solve_bracketed(Lov: torch.Tensor, Lp: torch.Tensor, orbitals: torch.
     status = torch.empty(np_, dtype=torch.int32, device=dev)
     bracket = torch.empty((np_, 2), dtype=torch.float64, device=dev)
     need = lib.cds_qp_workspace_bytes(nmo, nocc, M, np_, prec)
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     st = lib.cds_qp_solve_bracketed(nmo, nocc, M, _p(Lov), _p(Lp), _p(orb), np_, _p(eps),
                                     float(conv), int(max_iter), prec, _p(omega), _p(pole),
                                     _p(iters), _p(status), _p(bracket), _p(workspace),
@@ -595,8 +605,7 @@ def cds_sigma2_diag_cache(Lov: torch.Tensor, Lp: torch.Tensor, eps: torch.Tensor
     if cache is None or cache.numel() < cb:
         cache = torch.empty(max(cb, 1), dtype=torch.uint8, device=dev)
     need = lib.cds_sigma2_workspace_bytes(nmo, nocc, M, np_, nE, prec)
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     st = lib.cds_sigma2_diag_cache(nmo, nocc, M, _p(Lov), _p(Lp), np_, _p(eps), _p(E), nE, prec,
                                    _p(sigma), _p(dsigma), _p(cache), cache.numel(),
                                    _p(workspace), workspace.numel(), _stream(dev))
@@ -682,8 +691,7 @@ def cds_mp2_energy(Lov: torch.Tensor, eps: torch.Tensor, nocc: int, precision: s
     e_total = torch.empty(1, dtype=torch.float64, device=dev)
     e_pair = torch.empty(max(nocc, 1), dtype=torch.float64, device=dev)
     need = lib.cds_mp2_workspace_bytes(nmo, nocc, M, prec)
-    if workspace is None or workspace.numel() < need:
-        workspace = _workspace(need, dev)
+    workspace = _scratch(need, workspace, dev, precision == "fp64")
     st = lib.cds_mp2_energy(nmo, nocc, M, _p(Lov), _p(eps), prec, _p(e_pair), _p(e_total),
                             _p(workspace), workspace.numel(), _stream(dev))
     _check(st, "cds_mp2_energy")

@@ -636,6 +636,16 @@ static DxLayout dx_layout(void* ws, int32_t N, int32_t nmo, int32_t nocc, int32_
     return l;
 }
 
+// Vectors per batch: those of the other forms, fewer where they would take more than
+// kDxWorkspace bytes (from some 3,000 functions on).
+constexpr size_t kDxWorkspace = (size_t)4 << 30;
+static int32_t dx_batch(int32_t N, int32_t nmo, int32_t nocc, int32_t np, int32_t M) {
+    const size_t one = dx_layout(nullptr, N, nmo, nocc, np, 1).bytes;
+    const size_t two = dx_layout(nullptr, N, nmo, nocc, np, 2).bytes - one;
+    const size_t room = one < kDxWorkspace ? (kDxWorkspace - one) / std::max<size_t>(two, 1) : 0;
+    return (int32_t)std::min<size_t>(tr_batch(N, M), 1 + room);
+}
+
 static bool dx_serves(int32_t nbf, int32_t nmo, int32_t nocc, int32_t np) {
     return nbf >= kDxMinBasis && nbf <= (1 << 14) && nocc >= 0 && nocc <= nmo && nmo <= nbf &&
            np >= 0 && np <= 65535 && tc::device_ok();
@@ -645,9 +655,9 @@ static int cd_to_mo_fp64(int32_t N, int32_t nmo, int32_t nocc, int32_t M, const 
                          const double* C, const int32_t* orb, int32_t np, double* Lov, double* Lp,
                          void* ws, size_t ws_bytes, cudaStream_t stream) {
     const int32_t nv = nmo - nocc;
-    const int32_t kbx = tr_batch(N, M);
+    const int32_t kbx = dx_serves(N, nmo, nocc, np) ? dx_batch(N, nmo, nocc, np, M) : 0;
     // a workspace of the FP64-unit form's size is still served by that form
-    if (dx_serves(N, nmo, nocc, np) && ws_bytes >= dx_layout(nullptr, N, nmo, nocc, np, kbx).bytes) {
+    if (kbx > 0 && ws_bytes >= dx_layout(nullptr, N, nmo, nocc, np, kbx).bytes) {
         const DxLayout l = dx_layout(ws, N, nmo, nocc, np, kbx);
         const bool ov = nocc > 0 && nv > 0;
         CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
@@ -662,18 +672,13 @@ static int cd_to_mo_fp64(int32_t N, int32_t nmo, int32_t nocc, int32_t M, const 
         if (st) return st;
         for (int32_t K0 = 0; K0 < M; K0 += kbx) {
             const int32_t kb = std::min(kbx, M - K0);
-            auto sized = [](dx::Operand o, int64_t rows, int R) {
-                o.per = rows;
-                o.per_pad = dx::padded_rows(rows, R);
-                return o;
-            };
-            const dx::Operand tov = sized(l.tov, (int64_t)kb * nocc, dx::kRowsA);
-            const dx::Operand tp = sized(l.tp, (int64_t)kb * np, dx::kRowsA);
+            const dx::Operand tov = dx::sized(l.tov, (int64_t)kb * nocc, dx::kRowsA);
+            const dx::Operand tp = dx::sized(l.tp, (int64_t)kb * np, dx::kRowsA);
             const int64_t trow = (int64_t)kb * N;   // elements of T per r
             if (chain) {
                 st = dchain(L, N, K0, kb, C, nmo, nocc, orb, r0, nocc + np, l.T, stream);
             } else {
-                const dx::Operand u = sized(l.u, (int64_t)kb * N, dx::kRowsA);
+                const dx::Operand u = dx::sized(l.u, (int64_t)kb * N, dx::kRowsA);
                 const dx::PackedRows rows{L, npair_of(N), K0, N};
                 st = dx::slice(rows, u, dx::kRowsA, N, stream);
                 if (!st)
@@ -716,7 +721,7 @@ extern "C" size_t cds_cd_to_mo_workspace_bytes(int32_t nbf, int32_t nmo, int32_t
     const size_t least = cd_to_mo_least_bytes(nbf, nmo, nocc, M, np);
     return dx_serves(nbf, nmo, nocc, np)
                ? std::max(least, dx_layout(nullptr, nbf, nmo, nocc, np,
-                                           tr_batch(nbf, std::max(M, 1))).bytes)
+                                           dx_batch(nbf, nmo, nocc, np, std::max(M, 1))).bytes)
                : least;
 }
 

@@ -399,6 +399,9 @@ static int slice_any(const Src& src, const Operand& o, int R, int32_t kdim, cuda
 int slice(const RowMajor& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream) {
     return slice_any(src, o, R, kdim, stream);
 }
+int slice(const PanelRows& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream) {
+    return slice_any(src, o, R, kdim, stream);
+}
 int slice(const PackedRows& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream) {
     return slice_any(src, o, R, kdim, stream);
 }
@@ -693,6 +696,10 @@ static int gemm_any(const Operand& A, const SrcA& srca, const Operand& B, const 
 }
 
 int gemm(const Operand& A, const RowMajor& a, const Operand& B, const RowMajor& b, int32_t kdim, int64_t g0,
+         int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream) {
+    return gemm_any(A, a, B, b, kdim, g0, g1, out, active, err, stream);
+}
+int gemm(const Operand& A, const PanelRows& a, const Operand& B, const RowMajor& b, int32_t kdim, int64_t g0,
          int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream) {
     return gemm_any(A, a, B, b, kdim, g0, g1, out, active, err, stream);
 }

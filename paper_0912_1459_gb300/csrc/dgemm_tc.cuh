@@ -55,6 +55,13 @@ inline Operand carve(Carver& c, int64_t groups, int64_t per, int32_t kdim, int R
     return o;
 }
 
+// The same memory for another number of rows (at most those it was carved for).
+inline Operand sized(Operand o, int64_t rows, int R) {
+    o.per = rows;
+    o.per_pad = padded_rows(rows, R);
+    return o;
+}
+
 // Row sources: row(g, r)[k] is element k of row r of group g.  kAcross: neighbouring
 // rows, not neighbouring k, lie side by side in memory.
 struct RowMajor {         // x[(g gs + r) ld + k]
@@ -66,6 +73,15 @@ struct RowMajor {         // x[(g gs + r) ld + k]
         __device__ __forceinline__ double operator[](int k) const { return x[k]; }
     };
     __device__ __forceinline__ Row row(int64_t g, int64_t r) const { return {x + (g * gs + r) * ld}; }
+};
+struct PanelRows {        // row (j, a), a < an: x[(j nv + a) ld + k]
+    static constexpr bool kAcross = false;
+    const double* x;
+    int64_t nv, ld;
+    int32_t an;
+    __device__ __forceinline__ RowMajor::Row row(int64_t, int64_t r) const {
+        return {x + ((r / an) * nv + r % an) * ld};
+    }
 };
 struct PackedRows {       // rows (K, nu): A^K[nu][k] of the packed symmetric vectors
     static constexpr bool kAcross = false;
@@ -105,6 +121,7 @@ struct Columns {          // row j: C[k][col(j)], col(j) = j < nocc ? j : orb[j 
 
 // Slice an operand (R = kRowsA or kRowsB).
 int slice(const RowMajor& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
+int slice(const PanelRows& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
 int slice(const PackedRows& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
 int slice(const Columns& src, const Operand& o, int R, int32_t kdim, cudaStream_t stream);
 
@@ -116,6 +133,8 @@ struct Out {
     int64_t kdiv, m_hi, m_lo, g_s, n_s;
 };
 int gemm(const Operand& A, const RowMajor& a, const Operand& B, const RowMajor& b, int32_t kdim, int64_t g0,
+         int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream);
+int gemm(const Operand& A, const PanelRows& a, const Operand& B, const RowMajor& b, int32_t kdim, int64_t g0,
          int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream);
 int gemm(const Operand& A, const PackedRows& a, const Operand& B, const Columns& b, int32_t kdim, int64_t g0,
          int64_t g1, const Out& out, const int32_t* active, int32_t* err, cudaStream_t stream);

@@ -62,19 +62,21 @@ struct QpLayout {
     size_t bytes;
 };
 
-// least: the smallest workspace the solve works in, else the one it asks for.
+// have: a workspace of so many bytes, the self-energy's part of it what there is; 0: the one
+// to ask for.
 static QpLayout qp_layout(void* ws, int32_t nmo, int32_t nocc, int32_t M, int32_t np,
-                          int32_t precision, bool least = false) {
+                          int32_t precision, size_t have = 0) {
     Carver c(ws);
     QpLayout l;
     l.sig = c.take<double>(np);
     l.dsig = c.take<double>(np);
     l.active = c.take<int32_t>(np);
     l.nactive = c.take<int32_t>(1);
-    l.sigma_bytes = least ? sigma_ws_min_bytes(nmo, nocc, M, np, 1, precision)
-                          : sigma_ws_bytes(nmo, nocc, M, np, 1, precision);
+    const size_t head = c.off;
+    l.sigma_bytes = have ? (have > head ? have - head : 0)
+                         : sigma_ws_bytes(nmo, nocc, M, np, 1, precision);
     l.sigma_ws = c.take<char>(l.sigma_bytes);
-    l.bytes = c.off;
+    l.bytes = have ? head + l.sigma_bytes : c.off;
     return l;
 }
 
@@ -99,9 +101,10 @@ extern "C" int cds_qp_solve(int32_t nmo, int32_t nocc, int32_t M, const double* 
     if (precision != CDS_PREC_FP64 && !is_split_tc(precision)) return CDS_ERR_UNSUPPORTED;
     if (np == 0) return CDS_OK;
     if (!Lp || !orb || !eps || !omega || !pole || !iters || !status) return CDS_ERR_ARG;
-    QpLayout lay = qp_layout(workspace, nmo, nocc, M, np, precision);
-    if (workspace_bytes < lay.bytes) lay = qp_layout(workspace, nmo, nocc, M, np, precision, true);
-    if (!workspace || workspace_bytes < lay.bytes) return CDS_ERR_WORKSPACE;
+    if (!workspace || !workspace_bytes) return CDS_ERR_WORKSPACE;
+    const QpLayout lay = qp_layout(workspace, nmo, nocc, M, np, precision, workspace_bytes);
+    if (workspace_bytes < lay.bytes || !sigma_ws_ok(nmo, nocc, M, np, 1, precision, lay.sigma_bytes))
+        return CDS_ERR_WORKSPACE;
     int nb = (np + 127) / 128;
     k_qp_init<<<nb, 128, 0, stream>>>(eps, orb, np, nmo, omega, pole, iters, status, lay.active,
                                       lay.nactive);
@@ -319,9 +322,10 @@ extern "C" int cds_qp_solve_bracketed(int32_t nmo, int32_t nocc, int32_t M, cons
     if (np == 0) return CDS_OK;
     if (!Lp || !orb || !eps || !omega || !pole || !iters || !status || !bracket)
         return CDS_ERR_ARG;
-    QpLayout lay = qp_layout(workspace, nmo, nocc, M, np, precision);
-    if (workspace_bytes < lay.bytes) lay = qp_layout(workspace, nmo, nocc, M, np, precision, true);
-    if (!workspace || workspace_bytes < lay.bytes) return CDS_ERR_WORKSPACE;
+    if (!workspace || !workspace_bytes) return CDS_ERR_WORKSPACE;
+    const QpLayout lay = qp_layout(workspace, nmo, nocc, M, np, precision, workspace_bytes);
+    if (workspace_bytes < lay.bytes || !sigma_ws_ok(nmo, nocc, M, np, 1, precision, lay.sigma_bytes))
+        return CDS_ERR_WORKSPACE;
     int st = upload_brackets(nmo, nocc, np, orb, eps, bracket, stream);
     if (st) return st;
     const int nb = (np + 127) / 128;

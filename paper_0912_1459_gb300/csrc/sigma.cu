@@ -364,28 +364,26 @@ static int mp2_fp64(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, con
 static bool mp2_x_serves(int32_t nmo, int32_t nocc, int32_t M) {
     return M > 0 && sigma_x_serves(nmo, nocc, nocc);
 }
-// per-orbital sums (when the caller wants none) and the workspace of mp2_x
-static size_t mp2_ws_x(int32_t nmo, int32_t nocc, int32_t M) {
-    return align_up((size_t)nocc * sizeof(double)) + mp2_x_bytes(nmo, nocc, M);
-}
+// per-orbital sums (when the caller wants none), in front of the workspace of mp2_x
+static size_t mp2_pair_bytes(int32_t nocc) { return align_up((size_t)nocc * sizeof(double)); }
 
 size_t sigma_ws_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
                       int32_t precision) {
     if (precision == CDS_PREC_FP64) {
-        const size_t plain = fp64_part_bytes(nmo, nocc, np, nE);
-        return M > 0 && sigma_x_serves(nmo, nocc, np)
-                   ? std::max(plain, sigma_x_bytes(nmo, nocc, M, np, nE))
-                   : plain;
+        const size_t x = M > 0 && sigma_x_serves(nmo, nocc, np) ? sigma_x_bytes(nmo, nocc, M, np, nE) : 0;
+        return x ? x : fp64_part_bytes(nmo, nocc, np, nE);
     }
     if (is_split_tc(precision))
         return tc_workspace_bytes(nmo, nocc, M, np, nE, precision == CDS_PREC_TF32X3);
     return 0;
 }
 
-size_t sigma_ws_min_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
-                          int32_t precision) {
-    return precision == CDS_PREC_FP64 ? fp64_part_bytes(nmo, nocc, np, nE)
-                                      : sigma_ws_bytes(nmo, nocc, M, np, nE, precision);
+// Does a workspace of ws_bytes do?  FP64: also one of the fused kernel's size.
+bool sigma_ws_ok(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE, int32_t precision,
+                 size_t ws_bytes) {
+    if (precision != CDS_PREC_FP64) return ws_bytes >= sigma_ws_bytes(nmo, nocc, M, np, nE, precision);
+    return ws_bytes >= fp64_part_bytes(nmo, nocc, np, nE) ||
+           (M > 0 && sigma_x_serves(nmo, nocc, np) && sigma_x_fits(nmo, nocc, M, np, nE, ws_bytes));
 }
 
 int sigma2_dispatch(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* Lp,
@@ -396,9 +394,9 @@ int sigma2_dispatch(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, con
     if (precision == CDS_PREC_FP64) {
         // a workspace of the fused kernel's size is still served by that kernel
         if (M > 0 && sigma_x_serves(nmo, nocc, np) &&
-            ws_bytes >= sigma_x_bytes(nmo, nocc, M, np, nE))
+            sigma_x_fits(nmo, nocc, M, np, nE, ws_bytes))
             return sigma2_x(nmo, nocc, M, Lov, Lp, np, eps, E, nE, active, sigma, dsigma, ws,
-                            stream, resplit, static_cast<double*>(cache));
+                            ws_bytes, stream, resplit, static_cast<double*>(cache));
         return sigma2_fp64(nmo, nocc, M, Lov, Lp, np, eps, E, nE, active, sigma, dsigma,
                            static_cast<double*>(ws), stream, static_cast<double*>(cache));
     }
@@ -432,17 +430,17 @@ extern "C" int cds_sigma2_diag(int32_t nmo, int32_t nocc, int32_t M, const doubl
     if (precision != CDS_PREC_FP64 && !is_split_tc(precision)) return CDS_ERR_UNSUPPORTED;
     if (np == 0) return CDS_OK;
     if (!Lp || !eps || !E || !sigma || (nocc > 0 && nocc < nmo && !Lov)) return CDS_ERR_ARG;
-    size_t need = sigma_ws_min_bytes(nmo, nocc, M, np, nE, precision);
-    if (need && (!workspace || workspace_bytes < need)) return CDS_ERR_WORKSPACE;
+    const size_t have = workspace ? workspace_bytes : 0;
+    if (!sigma_ws_ok(nmo, nocc, M, np, nE, precision, have)) return CDS_ERR_WORKSPACE;
     return sigma2_dispatch(nmo, nocc, M, Lov, Lp, np, eps, E, nE, precision, nullptr, sigma,
-                           dsigma, workspace, workspace_bytes, stream);
+                           dsigma, workspace, have, stream);
 }
 
 extern "C" size_t cds_mp2_workspace_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t precision) {
     if (nmo <= 0 || nocc < 0 || nocc > nmo || M < 0) return 0;
     if (precision == CDS_PREC_FP64) {
-        const size_t plain = mp2_fp64_bytes(nmo, nocc);
-        return mp2_x_serves(nmo, nocc, M) ? std::max(plain, mp2_ws_x(nmo, nocc, M)) : plain;
+        const size_t x = mp2_x_serves(nmo, nocc, M) ? mp2_x_bytes(nmo, nocc, M) : 0;
+        return x ? mp2_pair_bytes(nocc) + x : mp2_fp64_bytes(nmo, nocc);
     }
     if (is_split16(precision)) return tc_mp2_workspace_bytes(nmo, nocc, M);
     return 0;
@@ -460,19 +458,19 @@ extern "C" int cds_mp2_energy(int32_t nmo, int32_t nocc, int32_t M, const double
         if (e_total) CDS_CUDA_TRY(cudaMemsetAsync(e_total, 0, sizeof(double), stream));
         return CDS_OK;
     }
-    const size_t need = precision == CDS_PREC_FP64
-                            ? mp2_fp64_bytes(nmo, nocc)
-                            : cds_mp2_workspace_bytes(nmo, nocc, M, precision);
-    if (!workspace || workspace_bytes < need) return CDS_ERR_WORKSPACE;
+    const size_t have = workspace ? workspace_bytes : 0;
     if (precision == CDS_PREC_FP64) {
-        if (mp2_x_serves(nmo, nocc, M) && workspace_bytes >= mp2_ws_x(nmo, nocc, M)) {
+        const size_t pair = mp2_pair_bytes(nocc), rest = have > pair ? have - pair : 0;
+        if (mp2_x_serves(nmo, nocc, M) && mp2_x_fits(nmo, nocc, M, rest)) {
             double* ep = e_pair ? e_pair : static_cast<double*>(workspace);
-            char* ws = static_cast<char*>(workspace) + align_up((size_t)nocc * sizeof(double));
-            const int st = mp2_x(nmo, nocc, M, Lov, eps, ep, ws, stream);
+            const int st = mp2_x(nmo, nocc, M, Lov, eps, ep, static_cast<char*>(workspace) + pair, rest, stream);
             return st ? st : sum_fixed(ep, nocc, e_total, stream);
         }
+        // a workspace of the fused kernel's size is still served by that kernel
+        if (have < mp2_fp64_bytes(nmo, nocc)) return CDS_ERR_WORKSPACE;
         return mp2_fp64(nmo, nocc, M, Lov, eps, e_pair, e_total, workspace, stream);
     }
+    if (!have || have < cds_mp2_workspace_bytes(nmo, nocc, M, precision)) return CDS_ERR_WORKSPACE;
     return mp2_tc(nmo, nocc, M, Lov, eps, precision, e_pair, e_total, workspace, stream);
 }
 
@@ -496,8 +494,8 @@ extern "C" int cds_sigma2_diag_cache(int32_t nmo, int32_t nocc, int32_t M, const
     if (!Lp || !eps || !E || !sigma || !cache || (nocc > 0 && nocc < nmo && !Lov))
         return CDS_ERR_ARG;
     if (cache_bytes < cds_sigma2_cache_bytes(nmo, nocc, np, precision)) return CDS_ERR_ARG;
-    size_t need = sigma_ws_min_bytes(nmo, nocc, M, np, nE, precision);
-    if (need && (!workspace || workspace_bytes < need)) return CDS_ERR_WORKSPACE;
+    const size_t have = workspace ? workspace_bytes : 0;
+    if (!sigma_ws_ok(nmo, nocc, M, np, nE, precision, have)) return CDS_ERR_WORKSPACE;
     return sigma2_dispatch(nmo, nocc, M, Lov, Lp, np, eps, E, nE, precision, nullptr, sigma,
-                           dsigma, workspace, workspace_bytes, stream, true, cache);
+                           dsigma, workspace, have, stream, true, cache);
 }

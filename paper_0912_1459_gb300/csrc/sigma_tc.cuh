@@ -81,9 +81,9 @@ inline bool is_split_tc(int32_t precision) {
 
 size_t sigma_ws_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
                       int32_t precision);
-// The least workspace sigma2_dispatch works in (FP64: that of the fused kernel).
-size_t sigma_ws_min_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
-                          int32_t precision);
+// Does sigma2_dispatch work in ws_bytes?  (FP64: also in less than sigma_ws_bytes.)
+bool sigma_ws_ok(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE, int32_t precision,
+                 size_t ws_bytes);
 
 int sigma2_dispatch(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* Lp,
                     int32_t np, const double* eps, const double* E, int32_t nE,

@@ -1,11 +1,16 @@
 // FP64 self-energy (paper Eq. SE) in two passes per group of orbitals:
 //   1. the MO integrals X^t[x][(j, b)] = sum_J Lp^J_tx Lov^J_jb of the group, an
-//      FP64-accurate tensor-core product (dgemm_tc.cu), into a scratch of at
-//      most kScratch bytes (0.8 GB for one orbital of an 840-function basis);
+//      FP64-accurate tensor-core product (dgemm_tc.cu), into a scratch of
+//      kScratch bytes or one orbital's integrals (0.8 GB at 840 functions);
 //   2. k_sigma_x: numerators (2 X_xy - X_yx) X_xy and the energy denominators.
 // The fused kernel this replaces formed the integrals with FP64 FMAs, which
 // the part issues at 2 a clock and SM: 0.14 s for an orbital of that basis.
 // Writing and reading the scratch costs 0.25 ms of HBM time per orbital.
+// Where that and the sliced factors (18 bytes per element of Lov and Lp) would take more
+// than kWorkspace bytes, or more than the caller's workspace, the spectators are taken in
+// panels, as many at once as fit: the virtual ones of the first sum, then the occupied
+// ones of the second, for each panel one orbital after another; the blocks add to
+// their partial sums from panel to panel.
 //
 // Pass 2 is bound by the FP64 pipe as well, so its energies are grouped.  For
 // a grid of more than kDirect energies with centre E0 and half width h, an
@@ -36,12 +41,13 @@ constexpr int part_stride(int32_t nE) { return nE == 1 ? 2 : nE <= kDirect ? kPa
 constexpr int kBlocks = 608;                // blocks of a launch: 4 per SM
 constexpr int kThreads = 256;
 constexpr int64_t kScratch = 512LL << 20;
+constexpr size_t kWorkspace = (size_t)4 << 30;   // asked for at most
 
 struct XTerm {
     int32_t nx, ns, nb, npb;
     int32_t xoff;              // row of x = 0 in an orbital's block of X
-    int64_t per;               // items per orbital
-    int64_t item0;             // first cached item of the term
+    int64_t per;               // items of a launch per orbital: the term's, or a panel's
+    int64_t item0, cper;       // cached items: first of the launch, per orbital
     int64_t cs, cy;            // column of (s, y): s cs + y cy
     const double *eps_s, *eps_x;
 };
@@ -55,6 +61,7 @@ struct XArgs {
     const int32_t* active;
     double* cache;             // numerators: written when X is given, else read
     double* part;
+    int32_t add;               // a later panel: add to the partial sums
 };
 
 // 1 / d: the PTX reciprocal seed and one cubic step (Newton's iteration with
@@ -172,7 +179,7 @@ k_sigma_x(const XArgs a) {
         const int x0 = A * TB + tr * 2, y0 = B * TB + tc * 2;
         double num[4], base[4];
         const double es = q.eps_s[s];
-        double* citem = a.cache ? a.cache + (q.item0 + (int64_t)t * q.per + r) * kItem + tid : nullptr;
+        double* citem = a.cache ? a.cache + (q.item0 + (int64_t)t * q.cper + r) * kItem + tid : nullptr;
         {
             const double* X = a.X + (int64_t)tl * a.tstride + (int64_t)s * q.cs;
             double exv[2], eyv[2];
@@ -284,13 +291,13 @@ k_sigma_x(const XArgs a) {
             double v = 0.0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) v += s_red[j][tid];
-            out[tid] = v;
+            out[tid] = a.add ? out[tid] + v : v;
         }
         for (int i = tid; i < 2 * ne; i += kThreads) {
             double v = 0.0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) v += s_sum[j][i];
-            out[kMom + i] = v;
+            out[kMom + i] = a.add ? out[kMom + i] + v : v;
         }
     } else {
         double* out = a.part + ((int64_t)t * gridDim.x + blockIdx.x) * (2 * NS);
@@ -305,7 +312,7 @@ k_sigma_x(const XArgs a) {
             double v = 0.0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) v += s_red[j][tid];
-            out[tid] = v;
+            out[tid] = a.add ? out[tid] + v : v;
         }
     }
 }
@@ -404,7 +411,7 @@ static void set_term(XTerm& q, int32_t nx, int32_t ns, int32_t xoff, int64_t cs,
     q.ns = ns;
     q.nb = nblocks_of(nx, TB);
     q.npb = (int32_t)npairs_of(q.nb);
-    q.per = nx > 0 && ns > 0 ? (int64_t)ns * q.npb : 0;
+    q.per = q.cper = nx > 0 && ns > 0 ? (int64_t)ns * q.npb : 0;
     q.xoff = xoff;
     q.cs = cs;
     q.cy = cy;
@@ -459,18 +466,23 @@ static int final_sum(const XArgs& a, int32_t np, int32_t nblk, const int32_t* er
 struct Layout {
     dx::Operand ov, p;
     double *X, *part;
-    int32_t* err;    // error word
+    int32_t* err;            // error word
     int32_t group, nblk;
+    // in panels (width[1] > 0): spectators of either sum held at once, their operand and X
+    int32_t width[2];
+    dx::Operand pan[2];
+    double* pX[2];
     size_t bytes;
 };
 
-// rows: rows of one orbital's block of X (all orbitals, or the virtual ones for MP2)
+// Everything at once.  rows: rows of one orbital's block of X (all orbitals, or the virtual
+// ones for MP2).
 static Layout layout(void* ws, int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE,
                      int32_t rows, int64_t items) {
     const int64_t ov = (int64_t)nocc * (nmo - nocc);
     // bulk copies want 16-byte addresses whatever the caller's workspace starts at
     Carver c(ws ? (void*)align_up((size_t)ws) : nullptr);
-    Layout l;
+    Layout l{};
     l.ov = dx::carve(c, 1, ov, M, dx::kRowsA);
     l.p = dx::carve(c, np, rows, M, dx::kRowsB);
     l.group = group_of(rows * ov, np);
@@ -481,6 +493,51 @@ static Layout layout(void* ws, int32_t nmo, int32_t nocc, int32_t M, int32_t np,
     l.err = c.take<int32_t>(1);
     l.bytes = c.off + 256;
     return l;
+}
+
+// One orbital and a panel of spectators at a time, panels of equal width and as wide as
+// `bytes` allow; .bytes = 0 where a panel of kPanelRows rows does not fit (narrower ones
+// leave the tensor cores idle, the fused kernel then serves).
+static Layout panel_layout(void* ws, size_t bytes, int32_t nmo, int32_t nocc, int32_t M, int32_t np,
+                           int32_t nE, bool mp2, int64_t items) {
+    constexpr int64_t kPanelRows = 1024;
+    const int32_t nv = nmo - nocc;
+    Carver c(ws ? (void*)align_up((size_t)ws) : nullptr);
+    Layout l{};
+    l.p = dx::carve(c, 1, mp2 ? nv : std::max(nocc, nv), M, dx::kRowsB);
+    l.group = 1;
+    l.nblk = blocks_of(items, 1);
+    const size_t nz = nE > kDirect ? (size_t)(nE + kZone - 1) / kZone : 1;
+    l.part = c.take<double>((size_t)np * nz * l.nblk * part_stride(nE));
+    l.err = c.take<int32_t>(1);
+    size_t most = 0;
+    for (int k = mp2 ? 1 : 0; k < 2; ++k) {
+        const int32_t total = k ? nocc : nv, nx = k ? nv : nocc;
+        auto take = [&](int32_t w) {         // both sums use the same memory in turn
+            Carver q = c;
+            l.pan[k] = dx::carve(q, 1, (int64_t)w * nx, M, dx::kRowsA);
+            l.pX[k] = q.take<double>((size_t)w * nx * nx);
+            return q.off + 256;
+        };
+        int32_t lo = 0, hi = total;          // the widest that fits
+        while (lo < hi) {
+            const int32_t mid = lo + (hi - lo + 1) / 2;
+            if (take(mid) <= bytes) lo = mid; else hi = mid - 1;
+        }
+        if (lo == 0 || (lo < total && (int64_t)lo * nx < kPanelRows)) return Layout{};
+        const int32_t n = (total + lo - 1) / lo;
+        l.width[k] = (total + n - 1) / n;
+        most = std::max(most, take(l.width[k]));
+    }
+    l.bytes = most;
+    return l;
+}
+
+// The layout for a workspace of `bytes` bytes; .bytes = 0: too small for either.
+static Layout layout_in(void* ws, size_t bytes, int32_t nmo, int32_t nocc, int32_t M, int32_t np,
+                        int32_t nE, bool mp2, int64_t items) {
+    const Layout l = layout(ws, nmo, nocc, M, np, nE, mp2 ? nmo - nocc : nmo, items);
+    return l.bytes <= bytes ? l : panel_layout(ws, bytes, nmo, nocc, M, np, nE, mp2, items);
 }
 
 // X of orbitals [t0, t0 + n).
@@ -502,27 +559,80 @@ bool sigma_x_serves(int32_t nmo, int32_t nocc, int32_t np) {
            tc::device_ok();
 }
 
-size_t sigma_x_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE) {
+static int64_t sigma_items(int32_t nmo, int32_t nocc, int32_t np) {
     XArgs a{};
     sigma_terms(a, nmo, nocc, np, nullptr);
-    return layout(nullptr, nmo, nocc, M, np, nE, nmo, a.tm[0].per + a.tm[1].per).bytes;
+    return a.tm[0].per + a.tm[1].per;
+}
+
+size_t sigma_x_bytes(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE) {
+    return layout_in(nullptr, kWorkspace, nmo, nocc, M, np, nE, false, sigma_items(nmo, nocc, np)).bytes;
+}
+
+bool sigma_x_fits(int32_t nmo, int32_t nocc, int32_t M, int32_t np, int32_t nE, size_t ws_bytes) {
+    return layout_in(nullptr, ws_bytes, nmo, nocc, M, np, nE, false, sigma_items(nmo, nocc, np)).bytes > 0;
+}
+
+// One sum's panel: spectators [s0, s0 + ns) of term k, whose columns of X are panel columns.
+static void set_panel(XArgs& a, const XArgs& all, int k, int32_t s0, int32_t ns) {
+    XTerm& q = a.tm[k];
+    a.tm[0].per = a.tm[1].per = 0;
+    a.tm[0].nb = a.tm[1].nb = 0;
+    q = all.tm[k];
+    q.ns = ns;
+    q.per = (int64_t)ns * q.npb;
+    q.item0 += (int64_t)s0 * q.npb;
+    q.eps_s += s0;
+    q.xoff = 0;
+    if (k == 0) q.cy = ns;           // columns (j, a)
+}
+
+// Orbitals [0, np) over the panels: q(t): the rows of orbital t's operand that a sum takes.
+template <typename Rows>
+static int panels(XArgs a, const Layout& l, int32_t nocc, int32_t nv, int32_t M, const double* Lov, int32_t np,
+                  Rows q, cudaStream_t stream) {
+    const XArgs all = a;
+    int st = CDS_OK;
+    bool first = true;
+    for (int k = l.width[0] > 0 ? 0 : 1; k < 2; ++k) {
+        const int32_t total = k ? nocc : nv, nx = k ? nv : nocc;
+        a.X = l.pX[k];
+        for (int32_t s0 = 0; s0 < total; s0 += l.width[k], first = false) {
+            const int32_t ns = std::min(l.width[k], total - s0);
+            const int64_t cols = (int64_t)ns * nx;
+            const dx::Operand A = dx::sized(l.pan[k], cols, dx::kRowsA);
+            const dx::PanelRows occ{Lov + (int64_t)s0 * M, nv, M, ns};
+            const dx::RowMajor vir{Lov + (int64_t)s0 * nv * M, 0, M};
+            st = k ? dx::slice(vir, A, dx::kRowsA, M, stream) : dx::slice(occ, A, dx::kRowsA, M, stream);
+            if (st) return st;
+            set_panel(a, all, k, s0, ns);
+            a.ncols = cols;
+            a.add = first ? 0 : 1;
+            for (int32_t t = 0; t < np; ++t) {
+                const dx::RowMajor b{q(t, k), 0, M};
+                const dx::Operand B = dx::sized(l.p, nx, dx::kRowsB);
+                const dx::Out out{l.pX[k], INT64_MAX, 0, 1, 0, cols};
+                const int32_t* on = a.active ? a.active + t : nullptr;
+                if ((st = dx::slice(b, B, dx::kRowsB, M, stream))) return st;
+                st = k ? dx::gemm(A, vir, B, b, M, 0, 1, out, on, l.err, stream)
+                       : dx::gemm(A, occ, B, b, M, 0, 1, out, on, l.err, stream);
+                if (st) return st;
+                a.t0 = t;
+                if ((st = eval(a, 1, l.nblk, false, stream))) return st;
+            }
+        }
+    }
+    return CDS_OK;
 }
 
 int sigma2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* Lp, int32_t np,
              const double* eps, const double* E, int32_t nE, const int32_t* active, double* sigma,
-             double* dsigma, void* ws, cudaStream_t stream, bool resplit, double* cache) {
+             double* dsigma, void* ws, size_t ws_bytes, cudaStream_t stream, bool resplit, double* cache) {
     const int64_t ov = (int64_t)nocc * (nmo - nocc);
     XArgs a{};
     sigma_terms(a, nmo, nocc, np, eps);
-    const Layout l = layout(ws, nmo, nocc, M, np, nE, nmo, a.tm[0].per + a.tm[1].per);
-    int st = CDS_OK;
-    if (resplit) {
-        CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
-        if ((st = dx::slice(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, stream)))
-            return st;
-        if ((st = dx::slice(dx::RowMajor{Lp, nmo, M}, l.p, dx::kRowsB, M, stream)))
-            return st;
-    }
+    const Layout l = layout_in(ws, ws_bytes, nmo, nocc, M, np, nE, false, a.tm[0].per + a.tm[1].per);
+    if (!l.bytes) return CDS_ERR_WORKSPACE;
     a.X = l.X;
     a.tstride = (int64_t)nmo * ov;
     a.ncols = ov;
@@ -531,6 +641,17 @@ int sigma2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const doub
     a.active = active;
     a.cache = cache;
     a.part = l.part;
+    int st = CDS_OK;
+    if (resplit || l.width[1] > 0) CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
+    if (l.width[1] > 0) {
+        st = panels(a, l, nocc, nmo - nocc, M, Lov, np,
+                    [&](int32_t t, int k) { return Lp + ((int64_t)t * nmo + (k ? nocc : 0)) * M; }, stream);
+        return st ? st : final_sum(a, np, l.nblk, l.err, sigma, dsigma, stream);
+    }
+    if (resplit) {
+        if ((st = dx::slice(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, stream))) return st;
+        if ((st = dx::slice(dx::RowMajor{Lp, nmo, M}, l.p, dx::kRowsB, M, stream))) return st;
+    }
     for (int32_t t0 = 0; t0 < np; t0 += l.group) {
         const int32_t n = std::min(l.group, np - t0);
         if (resplit || l.group < np)
@@ -539,14 +660,6 @@ int sigma2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const doub
         if ((st = eval(a, n, l.nblk, false, stream))) return st;
     }
     return final_sum(a, np, l.nblk, l.err, sigma, dsigma, stream);
-}
-
-size_t sigma_x_cached_bytes(int32_t nmo, int32_t nocc, int32_t np) {
-    XArgs a{};
-    sigma_terms(a, nmo, nocc, np, nullptr);
-    const int64_t ov = (int64_t)nocc * (nmo - nocc);
-    return align_up((size_t)np * blocks_of(a.tm[0].per + a.tm[1].per, group_of(nmo * ov, np)) *
-                    part_stride(1) * sizeof(double));
 }
 
 int sigma2_x_cached(int32_t nmo, int32_t nocc, int32_t np, const double* eps, const double* E,
@@ -573,30 +686,45 @@ static void mp2_terms(XArgs& a, int32_t nmo, int32_t nocc, const double* eps) {
     set_term(a.tm[1], nv, nocc, 0, nv, 1, eps, eps ? eps + nocc : nullptr);
 }
 
-size_t mp2_x_bytes(int32_t nmo, int32_t nocc, int32_t M) {
+static int64_t mp2_items(int32_t nmo, int32_t nocc) {
     XArgs a{};
     mp2_terms(a, nmo, nocc, nullptr);
-    return layout(nullptr, nmo, nocc, M, nocc, 1, nmo - nocc, a.tm[1].per).bytes;
+    return a.tm[1].per;
+}
+
+size_t mp2_x_bytes(int32_t nmo, int32_t nocc, int32_t M) {
+    return layout_in(nullptr, kWorkspace, nmo, nocc, M, nocc, 1, true, mp2_items(nmo, nocc)).bytes;
+}
+
+bool mp2_x_fits(int32_t nmo, int32_t nocc, int32_t M, size_t ws_bytes) {
+    return layout_in(nullptr, ws_bytes, nmo, nocc, M, nocc, 1, true, mp2_items(nmo, nocc)).bytes > 0;
 }
 
 int mp2_x(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const double* eps,
-          double* e_pair, void* ws, cudaStream_t stream) {
+          double* e_pair, void* ws, size_t ws_bytes, cudaStream_t stream) {
     const int32_t nv = nmo - nocc;
     const int64_t ov = (int64_t)nocc * nv;
     XArgs a{};
     mp2_terms(a, nmo, nocc, eps);
-    const Layout l = layout(ws, nmo, nocc, M, nocc, 1, nv, a.tm[1].per);
+    const Layout l = layout_in(ws, ws_bytes, nmo, nocc, M, nocc, 1, true, a.tm[1].per);
+    if (!l.bytes) return CDS_ERR_WORKSPACE;
     CDS_CUDA_TRY(cudaMemsetAsync(l.err, 0, sizeof(int32_t), stream));
-    int st = dx::slice(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, stream);
-    if (st) return st;
-    if ((st = dx::slice(dx::RowMajor{Lov, nv, M}, l.p, dx::kRowsB, M, stream)))
-        return st;
     a.X = l.X;
     a.tstride = (int64_t)nv * ov;
     a.ncols = ov;
     a.E = eps;
     a.nE = 1;
     a.part = l.part;
+    int st = CDS_OK;
+    if (l.width[1] > 0) {
+        st = panels(a, l, nocc, nv, M, Lov, nocc,
+                    [&](int32_t t, int) { return Lov + (int64_t)t * nv * M; }, stream);
+        return st ? st : final_sum(a, nocc, l.nblk, l.err, e_pair, nullptr, stream);
+    }
+    st = dx::slice(dx::RowMajor{Lov, 0, M}, l.ov, dx::kRowsA, M, stream);
+    if (st) return st;
+    if ((st = dx::slice(dx::RowMajor{Lov, nv, M}, l.p, dx::kRowsB, M, stream)))
+        return st;
     for (int32_t t0 = 0; t0 < nocc; t0 += l.group) {
         const int32_t n = std::min(l.group, nocc - t0);
         if ((st = integrals(l, ov, nv, M, Lov, Lov, t0, n, nullptr, stream))) return st;
