@@ -21,6 +21,7 @@
 // All kernels read a device control block and return at once after the
 // decomposition has stopped, so the host enqueues steps ahead and checks the
 // control block only every few steps.
+#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -1202,6 +1203,33 @@ static int sm_count() {
         return 152;
     return nsm;
 }
+// SMs that the kernels of `stream` may use: fewer than the device's in a green context (its
+// stream's, or the thread's).  A cooperative launch needs all of its CTAs on them at once.
+template <typename Fn>
+static Fn driver_fn(const char* name) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return ok ? (Fn)p : nullptr;
+}
+static int stream_sms(cudaStream_t stream) {
+    static const auto stream_green = driver_fn<decltype(&cuStreamGetGreenCtx)>("cuStreamGetGreenCtx");
+    static const auto green_res = driver_fn<decltype(&cuGreenCtxGetDevResource)>("cuGreenCtxGetDevResource");
+    static const auto current = driver_fn<decltype(&cuCtxGetCurrent)>("cuCtxGetCurrent");
+    static const auto ctx_res = driver_fn<decltype(&cuCtxGetDevResource)>("cuCtxGetDevResource");
+    int n = sm_count();
+    CUdevResource r{};
+    CUgreenCtx g = nullptr;
+    CUcontext c = nullptr;
+    if (stream_green && green_res && stream_green((CUstream)stream, &g) == CUDA_SUCCESS && g) {
+        if (green_res(g, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS) n = std::min(n, (int)r.sm.smCount);
+    } else if (current && ctx_res && current(&c) == CUDA_SUCCESS && c &&
+               ctx_res(c, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS) {
+        n = std::min(n, (int)r.sm.smCount);
+    }
+    return std::max(n, 1);
+}
 static int sel_blocks(int64_t n) { return (int)std::min<int64_t>(4 * 152, (n + kCdThreads - 1) / kCdThreads); }
 
 // Column capacity of the slice store for max_rank vectors.
@@ -1423,7 +1451,8 @@ static int cd_run_tc(int64_t n, int32_t max_rank, double* L, int32_t* piv, doubl
     // `count` passes, each the slicing, the projection GEMM and the steps up to
     // the next pass (everything reads its step from ctrl, and returns at once
     // after the decomposition has stopped)
-    const int step_sms = pipe_tr_ctas() > 0 && pipe_tr_ctas() < nsm ? nsm - pipe_tr_ctas() : nsm;
+    const int step_sms = std::min(stream_sms(stream),
+                                  pipe_tr_ctas() > 0 && pipe_tr_ctas() < nsm ? nsm - pipe_tr_ctas() : nsm);
     auto enqueue = [&](int count) -> int {
         for (int i = 0; i < count; ++i) {
             CDS_CUDA_TRY(launch_pdl(k_cd_project_tc, (unsigned)nres, kUpdThreads, 0, stream, nc,
@@ -1593,13 +1622,14 @@ int cd_decompose_run(int32_t nbf, const double* xyz, const double* alpha, const 
     CDS_LAUNCH_CHECK();
     CdCtrl h{};
     if (!df && !(on_chunk && *on_chunk) && direct_serves(n, max_rank)) {
-        // (a caller's workspace may be the size without its rows)
+        // (a caller's workspace may be the size without its rows, its stream may have fewer SMs)
         const CdLayout dl = cd_layout(workspace, nbf, false, false, max_rank, true);
-        if (workspace_bytes >= dl.bytes) {
+        const DirectShape sh = direct_shape(direct_sm_pairs(n));
+        if (workspace_bytes >= dl.bytes && direct_ctas(n, sh) <= stream_sms(stream)) {
             CdDirectArgs da{};
             da.n = n;
-            da.sh = direct_shape(direct_sm_pairs(n));
-            da.ctas = direct_ctas(n, da.sh);
+            da.sh = sh;
+            da.ctas = direct_ctas(n, sh);
             da.max_rank = max_rank;
             da.kcap = (int32_t)std::min<int64_t>(max_rank, n);
             da.L = L;
@@ -1949,9 +1979,9 @@ size_t cd_batch_direct_bytes(int32_t nmol, const BatchMol* mols) {
                          : align_up(sizeof(CdDirectArgs) * nmol) + align_up(16) +
                                align_up(kDirWordsRoom * sizeof(unsigned long long)) + align_up(rows);
 }
-static int cd_batch_direct(int32_t nmol, const BatchMol* mols, const std::vector<CdMol>& h,
-                           const CdCtrl* ctrl, int32_t* M_out, char* ws, cudaStream_t stream) {
-    const std::vector<DirectWave> waves = direct_waves(nmol, mols);
+static int cd_batch_direct(int32_t nmol, const BatchMol* mols, const std::vector<DirectWave>& waves,
+                           const std::vector<CdMol>& h, const CdCtrl* ctrl, int32_t* M_out, char* ws,
+                           cudaStream_t stream) {
     Carver top(ws);
     CdDirectArgs* table = top.take<CdDirectArgs>(nmol);
     int32_t* err = top.take<int32_t>(4);
@@ -2069,8 +2099,13 @@ int cd_batch_decompose(int32_t nmol, const BatchMol* mols, const BatchOffsets* o
     CDS_LAUNCH_CHECK();
     k_bcd_select<<<b_sel, kCdThreads, 0, stream>>>(lay.mols, nmol, 0);
     CDS_LAUNCH_CHECK();
-    if (!df && direct)
-        return cd_batch_direct(nmol, mols, h, lay.ctrl, M_out, static_cast<char*>(direct), stream);
+    if (!df && direct) {
+        const std::vector<DirectWave> waves = direct_waves(nmol, mols);
+        int most = 0;
+        for (const DirectWave& w : waves) most = std::max(most, w.ctas);
+        if (most <= stream_sms(stream))
+            return cd_batch_direct(nmol, mols, waves, h, lay.ctrl, M_out, static_cast<char*>(direct), stream);
+    }
     std::vector<CdCtrl> hc(nmol);
     for (int32_t k0 = 0; k0 <= kmax; k0 += kHostCheckEvery) {
         int32_t k1 = std::min(kmax, k0 + kHostCheckEvery);
