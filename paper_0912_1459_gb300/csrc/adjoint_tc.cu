@@ -128,18 +128,6 @@ struct GxArgs {
     void *ga_hi, *ga_lo, *gb_hi, *gb_lo;
 };
 
-// 1 / d to within 1 ulp: the PTX reciprocal seed and one cubic Newton step; zero,
-// subnormal, infinite and NaN d take the plain division.
-__device__ __forceinline__ double recip(double d) {
-    const uint32_t ex = ((uint32_t)__double2hiint(d) >> 20) & 0x7ffu;
-    if (ex - 2u >= 2042u) return 1.0 / d;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    e = fma(e, e, e);
-    return fma(r, e, r);
-}
-
 // Sums of four values over the warp (6 adds): lanes 8 i .. 8 i + 7 return value i.
 __device__ __forceinline__ double warp_sums4(const double (&v)[4]) {
     const int lane = threadIdx.x & 31;

@@ -119,6 +119,21 @@ __device__ __forceinline__ double double_of(float x) {
 // The double of a float pair.
 __device__ __forceinline__ double double_of(float2 v) { return double_of(v.x) + double_of(v.y); }
 
+// 1 / d within 1 ulp: the PTX reciprocal seed and one step of Newton's iteration with its
+// second-order term (the cubic Householder / Schulz step r (1 + e + e^2), e = 1 - d r), which
+// leaves the cube of the seed's error and two roundings.  d whose exponent, or whose
+// reciprocal's, is at the ends of the range (zero, subnormal, infinite, NaN among them)
+// takes the plain division.
+__device__ __forceinline__ double recip(double d) {
+    const uint32_t ex = ((uint32_t)__double2hiint(d) >> 20) & 0x7ffu;
+    if (ex - 2u >= 2042u) return 1.0 / d;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    double e = fma(-d, r, 1.0);
+    e = fma(e, e, e);
+    return fma(r, e, r);
+}
+
 // Decode a packed pair index I = nu(nu+1)/2 + mu into (mu, nu).
 __device__ __forceinline__ void unpack_pair(int64_t I, int32_t& mu, int32_t& nu) {
     double r = sqrt(8.0 * (double)I + 1.0);

@@ -29,6 +29,55 @@ constexpr int kRowsB = 64;    // rows per tile of a B operand
 constexpr int kStepK = 16;    // columns per k-step (one MMA k)
 constexpr int kDigits = 8;
 
+// (hi 2^32 + lo) 2^e as a double, rounded to nearest (ties to even).
+__device__ __forceinline__ double to_double(long long hi, long long lo, int e) {
+    unsigned long long l = (unsigned long long)lo + ((unsigned long long)hi << 32);
+    long long h = (hi >> 32) + (lo >> 63) + (l < (unsigned long long)lo ? 1 : 0);
+    const bool neg = h < 0;
+    if (neg) {
+        l = ~l + 1ull;
+        h = ~h + (l == 0 ? 1 : 0);
+    }
+    unsigned long long top = (unsigned long long)h, rest = l;
+    if (top == 0) { top = rest; rest = 0; e -= 64; }
+    if (top == 0) return 0.0;
+    const int lz = __clzll((long long)top);
+    if (lz) {
+        top = (top << lz) | (rest >> (64 - lz));
+        rest <<= lz;
+    }
+    // value = (top + rest 2^-64) 2^(64 - lz + e), top's leading bit set
+    unsigned long long mant = top >> 11;
+    const unsigned long long low = top & 0x7ffull;
+    const bool up = low > 0x400ull || (low == 0x400ull && (rest != 0 || (mant & 1ull)));
+    // exponent of the leading bit: 127 - lz + e; the mantissa's leading bit adds 1
+    const unsigned long long bexp = (unsigned long long)(127 - lz + e + 1023 - 1);
+    unsigned long long bits = (bexp << 52) + mant + (up ? 1ull : 0ull);
+    if (neg) bits |= 0x8000000000000000ull;
+    return __longlong_as_double((long long)bits);
+}
+
+// round(x 2^(62 - ex)), halves away from zero, for |x| < 2^ex.
+__device__ __forceinline__ long long fixed62(double x, int ex) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    int e = (int)((b >> 52) & 0x7ffull);
+    unsigned long long m = b & 0xfffffffffffffull;
+    if (e) m |= 1ull << 52;
+    else e = 1;
+    const int sh = e - 1013 - ex;   // q = m 2^sh, sh <= 9
+    if (sh >= 0) m <<= sh;
+    else if (sh > -54) m = (m + (1ull << (-sh - 1))) >> -sh;
+    else m = 0;
+    return (b >> 63) ? -(long long)m : (long long)m;
+}
+
+// BF16 bits of |x| 2^-ex, |x| < 2^ex, rounded down (0 below 2^-126).
+__device__ __forceinline__ uint32_t magnitude(double x, int ex) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7ffull) - 896 - ex;
+    return e > 0 ? ((uint32_t)e << 7) | ((uint32_t)(b >> 45) & 0x7fu) : 0u;
+}
+
 // One sliced operand: tiles of R rows, each [k-step][digit][R rows x 32
 // bytes], already in the order and 32-byte swizzle the MMA reads, so a k-step
 // of a tile is one contiguous bulk copy; mag the same with |x| / 2^ex in place of

@@ -64,19 +64,6 @@ struct XArgs {
     int32_t add;               // a later panel: add to the partial sums
 };
 
-// 1 / d: the PTX reciprocal seed and one cubic step (Newton's iteration with
-// the second-order term, r (1 + e + e^2), e = 1 - d r), within 1 ulp; zero,
-// subnormal, infinite and NaN d take the plain division.
-__device__ __forceinline__ double recip(double d) {
-    const uint32_t ex = ((uint32_t)__double2hiint(d) >> 20) & 0x7ffu;
-    if (ex - 2u >= 2042u) return 1.0 / d;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    e = fma(e, e, e);
-    return fma(r, e, r);
-}
-
 // Sum of each of N values over the warp with N - 1 + 5 - log2 N adds: value
 // index of a lane = its top log2 N lane bits (bit 4 first).
 template <int N>
