@@ -142,7 +142,11 @@ int cds_eri_columns(int32_t nbf, const double* xyz, const double* alpha,
 /* Workspace needed by cds_cd_decompose for a basis of nbf functions. */
 size_t cds_cd_workspace_bytes(int32_t nbf);
 
-/* Blocking.  precision: CDS_PREC_FP64 (binary64 throughout) or CDS_PREC_F32X2
+/* Blocking.  precision: CDS_PREC_FP64 (binary64 integrals, vectors and
+ * residuals; up to 768 pairs per SM and 4096 vectors the projections are exact
+ * integer sums over 56-bit copies of the vectors, off by at most sqrt(K) 2^-56 +
+ * K 2^-62 of the square roots of both pairs' initial diagonals, beyond that FP64
+ * sums) or CDS_PREC_F32X2
  * (the projections sum_K L^K_I L^K_P in float-pair arithmetic, ~2^-44 relative
  * per step, with the vectors held as float pairs while the decomposition runs;
  * integral columns, L^k, the residual diagonal and the pivot search stay FP64;

@@ -28,7 +28,7 @@
 // bounded (2 s of %globaltimer) and sets an error word instead of hanging.
 //
 // What bounds it: with few k the epilogue, until its conversions to FP64 (one a clock
-// and SM) became integer operations, 660 x 118,800 outputs of K = 896 0.81 -> 0.46 ms;
+// and SM) became integer operations, 660 x 118,800 outputs of K = 896 0.81 -> 0.42 ms;
 // with many k the shared memory's port, which the MMAs' operands and the TMA's writes
 // share: 640 clocks per k-block, 576 with the wide MMA below, for 384 of arithmetic
 // (5,280 x 896 of K = 118,800 2.55 ms, 1.3 PFLOP/s; tiles of 256 rows by pairs of CTAs,

@@ -1285,8 +1285,9 @@ static CdLayout cd_layout(void* ws, int32_t nbf, bool spec = true, bool tc = fal
 
 // Does the FP64 decomposition run as one launch (cd_direct.cuh)?  Its CTAs hold up
 // to 768 pairs each, and the pivot's rows in shared memory.  It is the faster form at
-// every size it holds (3.0x at 300 pairs, 2.2x at 28,920, 1.6x at 113,526); the launches
-// per step remain for what it does not hold, smaller workspaces and contracted shells.
+// every size it holds (2.9x at 300 pairs and 28,920, 1.7x at 113,526); the launches per step
+// remain for what it does not hold, smaller workspaces, streams with too few SMs for its
+// CTAs and contracted shells.
 static int direct_sms() { return std::min(sm_count(), kDirMaxCtas); }
 static int64_t direct_sm_pairs(int64_t n) { return (n + direct_sms() - 1) / direct_sms(); }
 static bool direct_serves(int64_t n, int32_t max_rank) {

@@ -11,24 +11,28 @@
 //  - the projections sum_K L^K_I L^K_P are taken in integers: beside its FP64 row
 //    every L^K_I is kept as a 56-bit number below the pair's scale 2^e > sqrt(D0_I)
 //    >= |L^K_I|, q = hi 2^26 + lo, and hi hi' and hi lo' + lo hi' are summed exactly
-//    in 64 bits (three 32-bit multiply-adds into 64 bits).  What is left out, the
-//    rounding of q and lo lo', is below 2^-56 of the scales' product for the whole
-//    sum (Cauchy-Schwarz: sum_K (L^K_I)^2 <= D0_I), where the FP64 chain rounds its
-//    partial sums, of up to that product, to 2^-53 each.  By the same bound
-//    |sum hi hi'| <= 2^60 and |sum hi lo'| <= 2^55 sqrt(K): no overflow;
+//    in 64 bits (three 32-bit multiply-adds into 64 bits).  In units of the scales'
+//    product the sum of K terms is off by at most sqrt(K) 2^-56 (the rounding of q, by
+//    Cauchy-Schwarz: sum_K (L^K_I)^2 <= D0_I) + K 2^-62 (lo lo', |lo| <= 2^25): 2^-51 at
+//    K = 400, 2^-49 at the largest K; unrelated digits leave about 2^-56 + sqrt(K) 2^-64.
+//    The FP64 chain may round its K partial sums to 2^-53 of that product each.  The
+//    vectors against extended precision, largest error before -> now: 300 pairs x 104
+//    2.8e-14 -> 2.3e-14, 1,176 x 139 9.1e-14 -> 5.5e-14, 1,830 x 117 (a chain of
+//    centres) 7.3e-14 -> 5.3e-14, 2,485 x 51 2.2e-13 -> 8.4e-14; rms and relative errors
+//    likewise.  No overflow: |sum hi hi'| <= 2^60, |sum hi lo'| <= 2^55 sqrt(K);
 //  - while one group of warps forms the integral column on the FP64 units, the
 //    others take the projections on the integer units;
 //  - the exchange of the residual maxima, the pivot choice and its ties are those
 //    of cd_steps.cuh: tagged words, one 128-byte line per CTA, every CTA decides.
 // Every wait is bounded and sets the error word instead of hanging.
-// Measured, whole decompositions, before -> now: 300 pairs x 104 vectors 1.93 -> 0.62
-// ms, 15,576 x 310 6.8 -> 2.7, 28,920 x 377 11.6 -> 4.6, 56,616 x 449 20.7 -> 10.8,
-// 113,526 x 411 29.0 -> 18.1.  A step of the third takes 10 us: 5 the projections (the
+// Measured, whole decompositions, a launch per step -> this: 300 pairs x 120 vectors 1.98
+// -> 0.68 ms, 15,576 x 293 6.5 -> 2.1, 28,920 x 372 11.0 -> 3.8, 56,616 x 456 21.2 -> 11.0,
+// 113,526 x 408 28.7 -> 17.2.  A step of the third takes 10 us: 5 the projections (the
 // 64-bit multiply-adds; the integral column beside them 3), 1 the block maxima, 2 the
 // exchange, 1 the choice of the pivot, 1 the pivot's data.  Rows beyond shared memory
 // come from L2: read upwards only, 41,616 x 452 took 17 ms, in turn 14, and with the
 // addresses advanced instead of formed anew 8.9.  Side by side, 100 molecules of 300
-// pairs 4.6 -> 3.1, 12 of 820 to 68,635 pairs 66 -> 48.
+// pairs 5.8 -> 3.5, 12 of 2,485 to 66,430 pairs 102 -> 72.
 #pragma once
 
 namespace cds {
@@ -52,7 +56,10 @@ inline DirectShape direct_shape(int64_t each) {   // at least `each` pairs per C
     s.per = (int)std::max<int64_t>(1, (each + kDirGroup - 1) / kDirGroup);
     s.width = (int)(((each + s.per - 1) / s.per + 31) / 32 * 32);
     s.pc = s.width * s.per;
-    // projection groups: enough threads to poll every line and to keep loads in flight
+    // Projection groups: enough threads to poll every line and to keep loads in flight, within
+    // the block's registers.  These / one / two / three everywhere: 28,920 pairs x 372 3.41 /
+    // 4.62 / 3.68 / 3.78 ms, 41,616 x 452 8.4 / 14.2 / 9.6 / 8.4, 5,050 x 200 1.00 / 1.10 / 0.99 /
+    // 0.97, 300 x 120 0.67 / 0.69 / 0.65 / 0.65.
     s.groups = s.width <= 64 ? 7 : s.width <= 96 ? 6 : s.width <= 128 ? 5 : s.width <= 192 ? 3 : 2;
     s.threads = s.width * (1 + s.groups) + 32;
     return s;

@@ -2,9 +2,10 @@
 // Eq. ps): FP64 path, the deterministic cross-tile reduction, and the entry
 // point that dispatches on precision.
 //
-// MO integrals are formed tile by tile from the factors (paper Sec. III:
-// recomputed from Eq. CD at every evaluation) and reduced with the energy
-// denominators in the same kernel; no o^2 v^2 integral array exists.
+// MO integrals are formed from the factors at every evaluation (paper Sec. III:
+// recomputed from Eq. CD).  The kernel here forms them tile by tile and reduces them
+// with the energy denominators at once; from 64 orbitals on those of a group of
+// orbitals, or of a panel of one's, are held in the workspace (sigma_x.cu).
 #include "sigma.cuh"
 #include "sigma_tc.cuh"
 #include "sigma_x.cuh"

@@ -1016,8 +1016,10 @@ int sigma2_tc(int32_t nmo, int32_t nocc, int32_t M, const double* Lov, const dou
         // with the numerators kept, the tensor-core epilogue evaluates the
         // first kGridSplitE energies and k_sigma_cached_grid the rest, at
         // the occupancy the epilogue warps of the tensor-core kernel lack
-        // (C60 shape, 20 orbitals x 64 energies: 43.6 ms against 52.6 ms
-        // with all energies in the epilogue)
+        // (C60 shape, 20 orbitals x 64 energies and Newton: 40.1 ms with one
+        // energy here, 48.8 / 47.7 / 45.0 with 4 / 8 / 16; the grid alone
+        // 43.6 against 52.6 ms with all of them, before the epilogue freed
+        // TMEM early)
         const bool split = cache && nE > kGridSplitE;
         if (split) P.nE_eval = kGridSplitE;
         const int nE_tc = split ? kGridSplitE : nE;   // picks the epilogue's energy chunk

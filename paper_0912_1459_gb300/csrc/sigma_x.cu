@@ -20,8 +20,8 @@
 // the Chebyshev expansion of a simple pole, so K moments sum n w v^k serve all
 // energies of the grid: 2 K + 18 FP64 operations per element instead of 7 per
 // element and energy.  K is chosen per 32 x 32 tile from the smallest |c| in it so
-// that the remainder is below 2^-56 (8 to 32 terms for |c| from 290 down to
-// 2.05); a tile with a pole nearer than that is evaluated energy by energy.
+// that the remainder is below 2^-56 (10 to 32 terms for |c| from 290 down to
+// 2.06); a tile with a pole nearer than that is evaluated energy by energy.
 #include "dgemm_tc.cuh"
 #include "sigma_x.cuh"
 #include "tcgen05.cuh"
